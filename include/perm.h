@@ -380,13 +380,27 @@ perm_status_t perm_scbs(int32_t k, int32_t *out);
 perm_status_t perm_alg2_launches(int64_t tau, int32_t n, int64_t *start, int64_t *delta, int64_t *end,
                                  int32_t max_launches, int32_t *count);
 
-/* The CUDA C++ source that the codegen engine would compile for A (for
-   inspection).  Writes at most cap bytes including the terminating NUL and
+/* The CUDA C++ source of the chained walk that the codegen engine generates for
+   A (for inspection; perm_elim_source gives the eliminated walk's, which runs
+   where it is cheaper).  Writes at most cap bytes including the terminating NUL and
    sets *len to the full length.  A kernel whose register spills exceed 512
    bytes per thread is rebuilt from the same text with a 255-register budget
    (__launch_bounds__(256, 1) in place of (256, 2)). */
 perm_status_t perm_codegen_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap,
                                   int64_t *len);
+
+/* The eliminated walk's kernel for A (for inspection): the sum over the low
+   columns of Sec. V's order distributes over the row products, so a generated
+   kernel walks only the outer columns in Gray order and sums out k low columns
+   at every step (every Gray index of the range is still accounted for).
+   Writes the source like perm_codegen_source, which gives the chained walk's
+   kernel; *len is 0 and *k is 0 where the chained walk runs instead (an explicit
+   order, split, chunk length or chain scheme, a deadline, a walk of zero
+   spans, or no column worth summing out).  order (n entries or NULL) gets the
+   outer columns by Gray position, then the k low columns, then the last
+   column. */
+perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap,
+                               int64_t *len, int32_t *k, int32_t *order);
 
 /* The matrix image that the precompiled generic kernels read for A (for
    inspection).  Sec. III names the sparse A and x as the two data

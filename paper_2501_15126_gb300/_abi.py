@@ -109,6 +109,8 @@ SIGNATURES = [
                                    ctypes.POINTER(c_i64), c_i32, ctypes.POINTER(c_i32)]),
     ("perm_codegen_source", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), ctypes.c_char_p, c_i64,
                                     ctypes.POINTER(c_i64)]),
+    ("perm_elim_source", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), ctypes.c_char_p, c_i64,
+                                 ctypes.POINTER(c_i64), ctypes.POINTER(c_i32), ctypes.POINTER(c_i32)]),
     ("perm_generic_image", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), c_vp, c_i64, ctypes.POINTER(c_i64),
                                    ctypes.POINTER(c_i32), ctypes.POINTER(c_i32), ctypes.POINTER(c_i32)]),
     ("perm_status_string", ctypes.c_char_p, [c_i32]),
@@ -270,6 +272,19 @@ def codegen_source(a, **kw) -> str:
     check(lib().perm_codegen_source(ctypes.byref(m.c), ctypes.byref(o), buf, n.value + 1, ctypes.byref(n)),
           "codegen")
     return buf.value.decode()
+
+
+def elim_source(a, **kw):
+    """perm_elim_source: (source, k, columns: outer by Gray position, low, last)."""
+    m = a if isinstance(a, CSRMatrix) else CSRMatrix(a)
+    o = opts(**kw)
+    n, k, order = c_i64(), c_i32(), (c_i32 * 64)()
+    check(lib().perm_elim_source(ctypes.byref(m.c), ctypes.byref(o), None, 0, ctypes.byref(n), ctypes.byref(k), order),
+          "perm_elim_source")
+    buf = ctypes.create_string_buffer(n.value + 1)
+    check(lib().perm_elim_source(ctypes.byref(m.c), ctypes.byref(o), buf, n.value + 1, ctypes.byref(n), None, None),
+          "perm_elim_source")
+    return buf.value.decode(), k.value, list(order)[: m.c.n]
 
 
 def generic_image(a, **kw):

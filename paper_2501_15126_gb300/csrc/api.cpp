@@ -338,6 +338,48 @@ perm_status_t choose_launch(perm_plan_s &P, int block_log2, int blocks_per_sm, i
     return PERM_OK;
 }
 
+// Low Gray bits over which [g_lo, g_hi) runs in full: the columns at those
+// positions take every setting inside the range, so their order is free.
+int range_free_cols(const perm_plan_s &P) {
+    int a = P.m.n - 1;
+    if (!P.subrange) return a;
+    if (P.g_lo) a = std::min(a, __builtin_ctzll(P.g_lo));
+    if (P.g_hi) a = std::min(a, __builtin_ctzll(P.g_hi));
+    return a;
+}
+
+// The eliminated walk replaces the chained one where the caller left the
+// walk to the library: an explicit order, split, chunk length, thread count
+// or chain scheme asks for the chained walk, and so does a deadline (its
+// tasks are sized and its stop is tested on that walk).
+bool elim_allowed(const perm_plan_s &P) {
+    const perm_opts_t &o = P.opts;
+    return P.m.n > 8 && !P.zero && (o.ordering == PERM_ORDER_AUTO || o.ordering == PERM_ORDER_SEARCH) &&
+           o.engine != PERM_ENGINE_XSHARED && !(o.flags & (PERM_FLAG_PAIRED_CHAIN | PERM_FLAG_PURE_REG)) &&
+           o.reg_rows <= 0 && o.shared_rows == 0 && o.chunk_log2 == 0 && o.threads == 0 && !(o.gr_ratio > 0) &&
+           o.timeout_ms == 0 && !codegen_no_fold();
+}
+
+// Chunks of 2^K outer steps: about eight tasks per resident warp, but at least
+// 2^3 steps (a start vector costs about as many updates as an eighth of a
+// step's program), unless that would leave resident warps without a task.
+void choose_launch_elim(perm_plan_s &P, int blocks_per_sm, int block) {
+    const int k = P.elim.k;
+    const uint64_t len = (P.g_hi - P.g_lo) >> k;
+    const double warps = (double)kSMCount * blocks_per_sm * (block / 32);
+    const int balance = floor_log2((uint64_t)std::max(1.0, (double)len / (32.0 * 8.0 * warps)));
+    const int fill = floor_log2((uint64_t)std::max(1.0, (double)len / (32.0 * warps)));
+    int K = std::max(balance, std::min(3, fill));
+    K = std::min({K, range_free_cols(P) - k, floor_log2(len)});
+    P.K = std::max(K, 0);
+    P.chunk_lo = (P.g_lo >> k) >> P.K;
+    P.chunk_hi = (P.g_hi >> k) >> P.K;
+    P.ntasks = (P.chunk_hi - P.chunk_lo + 31) / 32;
+    P.block = block;
+    P.grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)kSMCount * blocks_per_sm,
+                                                        ((int64_t)P.ntasks * 32 + block - 1) / block));
+}
+
 // The register rows requested by the caller, rounded down to whole groups.
 void split_for_rows(const Layout &L, int rows, int *k, int *c) {
     const int n = L.n;
@@ -405,6 +447,38 @@ static void codegen_layout(perm_plan_s &P) {
     }
 }
 
+// Plans the eliminated walk of a generated kernel (tables of at most
+// 2^max_width entries).  Walks whose zero spans skip most of the range keep
+// those: their chained walk drops 87-99.996 % of the steps.  Elsewhere the line is
+// half the chain's counted operations per Gray step: a step's program has no
+// block start, vote or skip, so equal counts would already be even, and dense
+// patterns (J_30: nothing to share) stay with the chain.  Measured, chained ->
+// eliminated: n=36 p=0.15 FP64 368 -> 2.76 ms per permanent (6.5 -> 0.024
+// operations per Gray step), n=34 p=0.2 0/1 7.0 -> 0.79 ms, 2^30-step slices of
+// the n=48 band: exact 6.41 -> 0.127 ms, FP64 16.9 -> 0.153 ms.
+void codegen_choose_elim(perm_plan_s &P, int max_width) {
+    P.use_elim = false;
+    if (max_width < 2 || !elim_allowed(P) || P.zero_spans) return;
+    ElimLimits lim;
+    lim.max_width = max_width;
+    const double range = std::log2((double)(P.g_hi - P.g_lo));
+    if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return;
+    if (P.elim.ops_per_step > 0.5 * P.ops_per_step) return;
+    P.use_elim = true;
+}
+
+// Switches a plan to (or from) the scales of the eliminated walk's sums.
+void adopt_elim(perm_plan_s &P) {
+    P.val_shift = P.use_elim ? P.elim.scale : 0;
+    if (!P.m.is_int)
+        P.abs_shift = P.use_elim ? P.elim.scale - P.m.n * elim_abs_bits(P.m.n, P.elim.k) : abs_shift_for(P.m);
+    if (!P.use_elim) return;
+    P.k = P.m.n;
+    P.c = P.m.n - 1;
+    P.k2 = 0;
+    P.ops_per_step = P.elim.ops_per_step;
+}
+
 perm_status_t plan_device_setup(perm_plan_s &P) {
     const int n = P.m.n;
     cudaError_t e;
@@ -469,8 +543,12 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
         std::string err;
         perm_status_t st = codegen_build(P, err);
         if (st != PERM_OK) return fail(st, err);
-        st = choose_launch(P, P.cg.block_log2, std::max(P.cg.blocks_per_sm, 1), P.cg.block);
-        if (st != PERM_OK) return st;
+        if (P.use_elim) {
+            choose_launch_elim(P, std::max(P.cg.blocks_per_sm, 1), P.cg.block);
+        } else {
+            st = choose_launch(P, P.cg.block_log2, std::max(P.cg.blocks_per_sm, 1), P.cg.block);
+            if (st != PERM_OK) return st;
+        }
         if (P.k + P.k2 < n) {
             const size_t bytes = (size_t)(n - P.k - P.k2) * (size_t)P.grid * P.block * (P.arith == 0 ? 8 : 4);
             if ((e = cudaMalloc(&P.d_xglob, bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc(x global rows)");
@@ -576,17 +654,18 @@ void describe(const perm_plan_s &P, perm_result_t *out) {
     out->reg_rows = P.engine == PERM_ENGINE_CODEGEN ? P.k : n;
     out->reg_cols = P.engine == PERM_ENGINE_CODEGEN ? P.c : n - 1;
     out->shared_rows = P.engine == PERM_ENGINE_CODEGEN ? P.k2 : 0;
-    out->chunk_log2 = P.K;
+    out->chunk_log2 = P.K + (P.use_elim ? P.elim.k : 0);
     out->threads = P.grid * P.block;
     out->regs_per_thread = P.regs;
     out->steps = P.zero ? 0 : P.g_hi - P.g_lo;
     out->ms_plan = P.ms_plan;
     out->ms_compile = P.ms_compile;
-    out->fp_ops_per_step = (P.engine == PERM_ENGINE_GENERIC && !P.direct && P.arith == 0 && P.m.n <= 32)
+    out->fp_ops_per_step = P.use_elim ? P.elim.ops_per_step
+                           : (P.engine == PERM_ENGINE_GENERIC && !P.direct && P.arith == 0 && P.m.n <= 32)
                                ? cost_per_step_dual(P.L, true)
                            : P.engine == PERM_ENGINE_XSHARED ? P.ops_per_step_paper   // a full product every step
                                                              : P.ops_per_step;
-    if (P.m.is_int && !P.zero) {   // integer multiply operations of the kernel that runs
+    if (P.m.is_int && !P.zero && !P.use_elim) {   // integer multiply operations of the kernel that runs
         const int fold = P.engine == PERM_ENGINE_CODEGEN ? (codegen_no_fold() ? 0 : 1) : (P.fold ? 2 : 0);
         out->fp_ops_per_step = ring_ops_per_step(P.m, P.L, P.limbs, fold);
     }
@@ -601,7 +680,7 @@ void describe(const perm_plan_s &P, perm_result_t *out) {
 // warp-wide, and lane 0 counts it once), out of ntasks 2^(K-B) warp blocks
 // (a range's idle lanes of its last task walk in step with the warp).
 double zero_skip_fraction(const perm_plan_s &P, uint64_t skipped) {
-    if (P.direct) return 0.0;
+    if (P.direct || P.use_elim) return 0.0;
     if (P.engine == PERM_ENGINE_XSHARED) return P.g_hi > P.g_lo ? (double)skipped / (double)(P.g_hi - P.g_lo) : 0.0;
     const int B = P.engine == PERM_ENGINE_GENERIC ? P.gf.block_log2 : P.cg.block_log2;
     const uint64_t warp_blocks = P.ntasks << std::max(0, P.K - B);
@@ -617,6 +696,8 @@ perm_status_t finish_raw(const perm_plan_s &P, const uint64_t *r, perm_result_t 
         std::memcpy(&lo, &r[1], 8);
         std::memcpy(&ab, &r[2], 8);
         ab = std::ldexp(ab, P.abs_shift);
+        hi = std::ldexp(hi, P.val_shift);
+        lo = std::ldexp(lo, P.val_shift);
         if (P.subrange) { out->f64 = hi; out->f64_lo = lo; out->abs_term_sum = ab; }
         else {
             const double f = (n % 2) ? 2.0 : -2.0;    // 4 (n mod 2) - 2, Algorithm 1
@@ -905,6 +986,31 @@ perm_status_t perm_codegen_source(const perm_matrix_t *A, const perm_opts_t *opt
     if (st != PERM_OK) return st;
     codegen_layout(P);
     std::string src = codegen_source(P);
+    if (len) *len = (int64_t)src.size();
+    if (buf && cap > 0) {
+        const size_t nb = std::min<size_t>((size_t)cap - 1, src.size());
+        std::memcpy(buf, src.data(), nb);
+        buf[nb] = 0;
+    }
+    return PERM_OK;
+}
+
+perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap, int64_t *len,
+                               int32_t *k, int32_t *outer) {
+    perm_plan_s P;
+    perm_status_t st = plan_prepare(A, opts, P);
+    if (st != PERM_OK) return st;
+    codegen_layout(P);
+    codegen_choose_elim(P, kElimWidth);
+    std::string src = P.use_elim ? elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs) : std::string();
+    adopt_elim(P);
+    if (k) *k = P.use_elim ? P.elim.k : 0;
+    if (outer)   // the outer columns by Gray position, the low columns, the last column
+        for (int i = 0; i < P.m.n; ++i)
+            outer[i] = !P.use_elim ? P.L.col_order[i]
+                       : i < P.elim.h ? P.elim.outer[i]
+                       : i < P.m.n - 1 ? P.elim.low[i - P.elim.h]
+                                       : P.elim.last;
     if (len) *len = (int64_t)src.size();
     if (buf && cap > 0) {
         const size_t nb = std::min<size_t>((size_t)cap - 1, src.size());

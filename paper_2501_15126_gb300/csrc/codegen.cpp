@@ -688,53 +688,78 @@ perm_status_t same_on_probe(const perm_plan_s &P, const CacheEntry &a, const Cac
 perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
     Driver &d = driver();
     if (!d.ok) { err = "CUDA driver entry points unavailable"; return PERM_ERR_CUDA; }
-    const std::string src = codegen_source(P);
-    P.cg.block = kCodegenBlock;
-    P.cg.block_log2 = codegen_block_log2(P);
     const bool use_cache = !(P.opts.flags & PERM_FLAG_NO_KERNEL_CACHE);
     // a module belongs to one device's context: the cache key names the device
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); dev = -1; }
-    const std::string key = "device " + std::to_string(dev) + "\n" + src;
-    if (use_cache) {
-        std::lock_guard<std::mutex> lk(g_cache_mu);
-        auto it = g_cache.find(key);
-        if (it != g_cache.end()) {
-            P.cg.module = it->second.module;
-            P.cg.function = it->second.function;
-            P.cg.regs = it->second.regs;
-            P.cg.blocks_per_sm = it->second.blocks_per_sm;
-            P.cg.cached = true;
-            P.regs = P.cg.regs;
-            P.ms_compile = 0.0;
-            return PERM_OK;
-        }
-    }
+    P.cg.block = kCodegenBlock;
+    P.cg.block_log2 = codegen_block_log2(P);
     const double t0 = now_ms();
     CacheEntry ce;
-    perm_status_t st = compile_and_load(src, ce, err, P.xs_bytes());
-    if (st != PERM_OK) return st;
-    const bool fixed_budget = std::getenv("PERM_CODEGEN_MIN_BLOCKS") != nullptr;
-    if (ce.local_bytes > kMaxLocalFrame && !fixed_budget && codegen_min_blocks(P) > 1) {
-        if (driver().moduleUnload) driver().moduleUnload(ce.module);
-        ce = CacheEntry();
-        Emitter e1(P, 1);
-        st = compile_and_load(e1.emit(), ce, err, P.xs_bytes());
+    std::string key;
+    auto cached = [&](const std::string &src) {
+        key = "device " + std::to_string(dev) + "\n" + src;
+        if (!use_cache) return false;
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        auto it = g_cache.find(key);
+        if (it == g_cache.end()) return false;
+        P.cg.module = it->second.module;
+        P.cg.function = it->second.function;
+        P.cg.regs = it->second.regs;
+        P.cg.blocks_per_sm = it->second.blocks_per_sm;
+        P.cg.cached = true;
+        P.regs = P.cg.regs;
+        P.ms_compile = 0.0;
+        return true;
+    };
+    // The eliminated walk, planned narrower while its kernel spills (255
+    // registers): FP64 steps tolerate a small frame (the FP64 pipe bounds
+    // them), exact ones none; then the chained walk.
+    perm_status_t st = PERM_OK;
+    bool built = false;
+    for (int width = kElimWidth; width >= 2 && !built; --width) {
+        codegen_choose_elim(P, width);
+        if (!P.use_elim) break;
+        const std::string src = elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs);
+        if (cached(src)) { adopt_elim(P); return PERM_OK; }
+        st = compile_and_load(src, ce, err, 0);
         if (st != PERM_OK) return st;
-    } else if (P.arith != 0 && ce.local_bytes > 0 && !fixed_budget) {
-        // exact kernel with any spills: cross-check against the 255-register build
-        CacheEntry wide;
-        Emitter e1(P, 1);
-        st = compile_and_load(e1.emit(), wide, err, P.xs_bytes());
-        if (st != PERM_OK) { driver().moduleUnload(ce.module); return st; }
-        bool same = false;
-        st = same_on_probe(P, ce, wide, &same, err);
-        if (st != PERM_OK) { driver().moduleUnload(ce.module); driver().moduleUnload(wide.module); return st; }
-        if (same) {
-            driver().moduleUnload(wide.module);
+        if (ce.local_bytes <= (P.arith == 0 ? kMaxLocalFrame : 0)) {
+            built = true;
         } else {
             driver().moduleUnload(ce.module);
-            ce = wide;
+            ce = CacheEntry();
+        }
+    }
+    P.use_elim = built;
+    adopt_elim(P);
+    if (!built) {
+        const std::string src = codegen_source(P);
+        if (cached(src)) return PERM_OK;
+        st = compile_and_load(src, ce, err, P.xs_bytes());
+        if (st != PERM_OK) return st;
+        const bool fixed_budget = std::getenv("PERM_CODEGEN_MIN_BLOCKS") != nullptr;
+        if (ce.local_bytes > kMaxLocalFrame && !fixed_budget && codegen_min_blocks(P) > 1) {
+            if (driver().moduleUnload) driver().moduleUnload(ce.module);
+            ce = CacheEntry();
+            Emitter e1(P, 1);
+            st = compile_and_load(e1.emit(), ce, err, P.xs_bytes());
+            if (st != PERM_OK) return st;
+        } else if (P.arith != 0 && ce.local_bytes > 0 && !fixed_budget) {
+            // exact kernel with any spills: cross-check against the 255-register build
+            CacheEntry wide;
+            Emitter e1(P, 1);
+            st = compile_and_load(e1.emit(), wide, err, P.xs_bytes());
+            if (st != PERM_OK) { driver().moduleUnload(ce.module); return st; }
+            bool same = false;
+            st = same_on_probe(P, ce, wide, &same, err);
+            if (st != PERM_OK) { driver().moduleUnload(ce.module); driver().moduleUnload(wide.module); return st; }
+            if (same) {
+                driver().moduleUnload(wide.module);
+            } else {
+                driver().moduleUnload(ce.module);
+                ce = wide;
+            }
         }
     }
     P.ms_compile = now_ms() - t0;

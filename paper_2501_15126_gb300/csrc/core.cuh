@@ -357,6 +357,67 @@ __device__ __forceinline__ void ring_sub<2>(Ring<2> &a, const Ring<2> &b) {
     a.w[1] = (u32)(v >> 32);
 }
 
+// ------------------------------------------------------------------ ring helpers of the eliminated walk
+// A signed 64-bit value as a ring element, and products of a ring element
+// with a 32-bit, a 64-bit and a ring factor (two's complement, modulo 2^(32 L)).
+template <int L>
+__device__ __forceinline__ Ring<L> ring_of(i64 v) {
+    Ring<L> r;
+    const u32 sign = v < 0 ? 0xffffffffu : 0u;
+#pragma unroll
+    for (int i = 0; i < L; ++i) r.w[i] = i == 0 ? (u32)(u64)v : i == 1 ? (u32)((u64)v >> 32) : sign;
+    return r;
+}
+template <int L>
+__device__ __forceinline__ Ring<L> ring_times(const Ring<L> &q, int x) { return ring_mul<L>(q, x); }
+template <int L>
+__device__ __forceinline__ Ring<L> ring_times(const Ring<L> &q, i64 x) {
+    // x = lo + 2^32 hi - 2^64 [x < 0] with lo, hi unsigned 32-bit words
+    const u32 f[2] = {(u32)(u64)x, (u32)((u64)x >> 32)};
+    Ring<L> r;
+#pragma unroll
+    for (int i = 0; i < L; ++i) r.w[i] = 0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        u64 c = 0;
+#pragma unroll
+        for (int i = 0; i + k < L; ++i) {
+            const u64 t = (u64)q.w[i] * f[k] + r.w[i + k] + c;
+            r.w[i + k] = (u32)t;
+            c = t >> 32;
+        }
+    }
+    if (x < 0) {
+        u32 borrow = 0;
+#pragma unroll
+        for (int i = 2; i < L; ++i) {
+            const u64 t = (u64)r.w[i] - (u64)q.w[i - 2] - (u64)borrow;
+            r.w[i] = (u32)t;
+            borrow = (u32)(t >> 63);
+        }
+    }
+    return r;
+}
+template <int L>
+__device__ __forceinline__ Ring<L> ring_times(const Ring<L> &q, const Ring<L> &x) {
+    Ring<L> r;
+#pragma unroll
+    for (int i = 0; i < L; ++i) r.w[i] = 0;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        u64 c = 0;
+#pragma unroll
+        for (int i = 0; i + k < L; ++i) {
+            const u64 t = (u64)q.w[i] * x.w[k] + r.w[i + k] + c;
+            r.w[i + k] = (u32)t;
+            c = t >> 32;
+        }
+    }
+    return r;
+}
+template <int L>
+__device__ __forceinline__ Ring<L> ring_minus(Ring<L> a, const Ring<L> &b) { ring_sub<L>(a, b); return a; }
+
 // Exact arithmetic in Z / 2^(32 NL): NL 32-bit limbs, stored and reduced as
 // ceil(NL/2) 64-bit words (an odd limb count leaves the top half-word of the
 // last word zero; sums of stored words stay right modulo 2^(32 NL)).
@@ -778,6 +839,56 @@ __device__ __forceinline__ void walk_tasks(Pol &pol, const WalkArgs &wa) {
     }
     // the warp's skipped blocks (a skip is warp-wide: one count per warp block)
     if (wa.skip_counter && lane == 0 && skipped) atomicAdd(wa.skip_counter, skipped);
+}
+
+// ------------------------------------------------------------------ the eliminated walk
+// A Gray walk over the outer columns only: the policy's step() adds the
+// signed sum of the terms of all 2^k settings of its k low columns (summed out
+// by a straight-line program, elim.hpp) to the block accumulator.  q, K and the
+// task's chunk indices count outer Gray indices; the sign of outer index g is
+// (-1)^g, as in the plain walk.  A step is hundreds of operations, so the flip
+// between two steps is a run-time switch, like a block boundary's.
+template <class Pol, class A>
+__device__ __forceinline__ typename A::Acc walk_chunk_elim(u64 q, int K) {
+    typename A::X x[Pol::NX];
+    const u64 g0 = q << K;
+    Pol::init_x(x, g0 ^ (g0 >> 1));
+    typename A::Acc acc = A::acc_zero();
+    typename A::Blk mid = A::blk_zero();
+    const u64 len = 1ull << K;
+    u64 l = 0;
+    for (;;) {
+        Pol::step(x, mid, ((g0 + l) & 1ull) != 0);
+        if (++l >= len) break;
+        if ((l & 7) == 0) {   // merged into the compensated accumulator every 8 steps
+            A::acc_merge(acc, mid);
+            mid = A::blk_zero();
+        }
+        const int j = ctz64(l);   // the same column in every lane; only column K-1's sign differs (Lemma 1)
+        Pol::flip_dyn(j, x, (((g0 + l) >> (j + 1)) & 1ull) ? -1 : 1);
+        __syncwarp();
+    }
+    A::acc_merge(acc, mid);
+    return acc;
+}
+
+template <class Pol, class A>
+__device__ __forceinline__ void elim_tasks(const WalkArgs &wa) {
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        u64 task = 0;
+        if (lane == 0) task = past_deadline(wa.timeout_ns, wa.deadline_word, wa.abort_flag) ? ~0ull : atomicAdd(wa.task_counter, 1ull);
+        task = __shfl_sync(PERM_FULLMASK, task, 0);
+        if (task >= wa.ntasks) break;
+        u64 q = wa.chunk_lo + task * 32ull + (u64)lane;
+        const bool live = q < wa.chunk_hi;
+        if (!live) q = wa.chunk_hi - 1;     // idle lanes shadow a real chunk to stay in step
+        typename A::Acc acc = walk_chunk_elim<Pol, A>(q, wa.K);
+        if (!live) acc = A::acc_zero();
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
+        if (lane == 0) A::acc_store(wa.task_out + task * (u64)A::ACC_WORDS, acc);
+    }
 }
 
 // ------------------------------------------------------------------ final reduction

@@ -1,0 +1,76 @@
+// elim.hpp -- the eliminated walk: a Gray walk over the outer columns whose
+// every step sums the terms of all 2^k settings of k low columns at once.
+//
+// The Nijenhuis-Wilf sum (Eq. 2, Sec. II) runs over the subsets S of the
+// first n-1 columns, sum_S (-1)^|S| prod_i x_i(S).  Row i's factor depends only
+// on the columns that touch row i, so for sparse matrices the sum over the low
+// columns distributes over the product: with the outer columns fixed, each row
+// is a table over the settings of the low columns that touch it (x_i plus a
+// subset of their entries), and a low column is summed out by multiplying the
+// tables that mention it and subtracting the column-on half from the
+// column-off half.  Every Gray index of the range is still accounted for, and
+// every term is the same product of n numbers; products and sums shared
+// between terms are formed once.  The paired and two-state chains (core.cuh)
+// are the k = 1 case; Sec. V's reuse of a global product is the case of rows
+// that no low column touches.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+#include <string>
+#include <vector>
+
+#include "host.hpp"
+
+namespace perm {
+
+// One operation of a step's program.  Values are numbered 0..n-1 (x of the
+// original rows) and then one per operation.
+enum ElimKind : uint8_t {
+    kElimAdd = 0,      // v = value a + entry (row b, column c)
+    kElimMul = 1,      // v = a * b
+    kElimMulSub = 2,   // v = c - a * b
+    kElimSub = 3       // v = a - b
+};
+
+struct ElimOp {
+    uint8_t kind;
+    int32_t a, b, c;
+};
+
+struct ElimPlan {
+    int n = 0, k = 0, h = 0;          // k low columns summed out, h outer columns walked
+    int low[kNMax] = {};              // low columns in elimination order (original indices)
+    int outer[kNMax] = {};            // outer column at Gray position p (original index)
+    int last = 0;                     // the column that never flips
+    int exp2[kNMax] = {};             // FP64: row i is walked as x_i 2^-exp2[i] (exact scaling, |x_i| <= 1)
+    int scale = 0;                    // FP64: sum of exp2: the walk's sum times 2^scale is the true one
+    std::vector<ElimOp> ops;
+    int result = 0;                   // the value that holds the step's signed sum
+    std::vector<double> bound;        // exact: a bound of each value's magnitude (n + ops entries)
+    double ops_per_step = 0.0;        // counted operations per Gray step, flips and accumulation included
+};
+
+struct ElimLimits {
+    int max_width = 5;                // tables of at most 2^max_width entries while a column is summed out
+    int max_ops = 1200;               // operations of a step's program
+    double full_blocks = 19456.0;     // outer steps that fill the GPU: fewer take as long as these
+    int candidates = kNMax;           // low columns tried per round of the search
+};
+
+// Picks the low columns among the first `free_cols` positions of col_order
+// (over which the walked range runs in full) and writes the step's program.
+// range_log2: log2 of the number of Gray indices walked.  False when no
+// column is worth summing out.
+bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double range_log2, const ElimLimits &lim,
+               ElimPlan &out);
+
+// The FP32 sum of |terms| walks every row's magnitude 2^bits above |x_i| <= 1,
+// so that a product of n of them, summed over 2^(k+3) terms, neither overflows
+// nor drifts into FP32's subnormals.
+inline int elim_abs_bits(int n, int k) { return std::max(0, std::min(8, (120 - k) / n)); }
+
+// The CUDA C++ of the generated kernel (limbs 0: FP64, else the exact ring).
+std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want_abs);
+
+}  // namespace perm

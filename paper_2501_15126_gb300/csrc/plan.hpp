@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "codegen.hpp"
+#include "elim.hpp"
 #include "host.hpp"
 #include "kernels.hpp"
 
@@ -55,6 +56,9 @@ struct perm_plan_s {
     bool zero_spans = false;  // codegen: the kernel widens zero skips into zero spans (core.cuh)
     bool want_abs = true;     // FP64 walks: accumulate sum|terms| (generated kernels: see codegen_layout)
     int abs_shift = 0;        // FP64 / double-double: sum|terms| is accumulated as sum|terms| 2^-abs_shift
+    bool use_elim = false;    // the walk sums out low columns (elim.hpp); chunks count outer Gray indices
+    perm::ElimPlan elim;
+    int val_shift = 0;        // FP64: the walk's sum is the true one times 2^-val_shift
     int kind() const { return dd ? perm::kKindDD : 2 * limbs + (fold ? 1 : 0); }   // generic kernel family
     int img_kind() const { return dd ? perm::kImgDD : (arith ? perm::kImgInt : perm::kImgF64); }   // matrix image layout
     uint64_t total = 0;       // 2^(n-1)
@@ -128,5 +132,13 @@ void build_devmat_into(const Matrix &m, const Layout &L, int img, int nmax, unsi
 perm_matrix_t matrix_view(const Matrix &m, std::vector<int32_t> &ptr, std::vector<int32_t> &idx,
                           std::vector<unsigned char> &vals);
 perm_status_t choose_launch(perm_plan_s &P, int block_log2, int blocks_per_sm, int block);
+// The eliminated walk: whether the call may take it, its column plan, and its
+// chunks and grid.
+bool elim_allowed(const perm_plan_s &P);
+int range_free_cols(const perm_plan_s &P);
+constexpr int kElimWidth = 5;   // generated kernels: tables of at most 2^5 entries
+void codegen_choose_elim(perm_plan_s &P, int max_width);
+void adopt_elim(perm_plan_s &P);
+void choose_launch_elim(perm_plan_s &P, int blocks_per_sm, int block);
 
 }  // namespace perm
