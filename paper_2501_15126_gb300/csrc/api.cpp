@@ -636,7 +636,7 @@ perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
         e = debug_fail(kSiteLaunch) ? cudaErrorLaunchFailure : codegen_launch(P, wa, st);
         if (e != cudaSuccess) return cuda_fail(e, "walk kernel launch");
     }
-    if ((e = reduce_launch(P.arith, task_out, P.ntasks, P.d_ws + 2, st)) != cudaSuccess)
+    if ((e = reduce_launch(P.arith, task_out, P.ntasks, P.d_ws + 2, P.d_ws + kWsReduced, st)) != cudaSuccess)
         return cuda_fail(e, "reduce kernel launch");
     if (record_events && (e = cudaEventRecord(P.ev1, st)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
     if ((e = cudaMemcpyAsync(P.h_res, P.d_ws, 8 * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess)

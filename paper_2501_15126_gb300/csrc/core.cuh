@@ -165,15 +165,25 @@ struct ArithF64 {
         a.lo += e;
         a.abs += (double)b.a;
     }
+    // The sum of two accumulators, left unnormalised: in a tree of these only the
+    // high parts wait on one another (one addition per level, where normalising
+    // every level made a chain of nine); acc_norm ends the tree.
     static __device__ __forceinline__ Acc acc_add(Acc a, Acc b) {
-        double s = a.hi + b.hi;
-        double bb = s - a.hi;
-        double e = (a.hi - (s - bb)) + (b.hi - bb);
-        e += a.lo + b.lo;
+        const double s = a.hi + b.hi;
+        const double bb = s - a.hi;
+        const double e = (a.hi - (s - bb)) + (b.hi - bb);
         Acc r;
-        r.hi = s + e;
-        r.lo = e - (r.hi - s);
+        r.hi = s;
+        r.lo = e + (a.lo + b.lo);
         r.abs = a.abs + b.abs;
+        return r;
+    }
+    static __device__ __forceinline__ Acc acc_norm(Acc a) {
+        Acc r;
+        r.hi = a.hi + a.lo;
+        const double bb = r.hi - a.hi;
+        r.lo = (a.hi - (r.hi - bb)) + (a.lo - bb);
+        r.abs = a.abs;
         return r;
     }
     static __device__ __forceinline__ Acc shfl_down(Acc a, int d) {
@@ -274,6 +284,7 @@ struct ArithDD {
         a.abs += (double)b.a;
     }
     static __device__ __forceinline__ Acc acc_add(Acc a, Acc b) { return ArithF64::acc_add(a, b); }
+    static __device__ __forceinline__ Acc acc_norm(Acc a) { return ArithF64::acc_norm(a); }
     static __device__ __forceinline__ Acc shfl_down(Acc a, int d) { return ArithF64::shfl_down(a, d); }
     static constexpr int ACC_WORDS = ArithF64::ACC_WORDS;
     static __device__ __forceinline__ void acc_store(u64 *dst, Acc a) { ArithF64::acc_store(dst, a); }
@@ -465,6 +476,7 @@ struct ArithExact {
     static __device__ __forceinline__ Acc acc_zero() { return blk_zero(); }
     static __device__ __forceinline__ void acc_merge(Acc &a, const Blk &b) { ring_add<L>(a, b); }
     static __device__ __forceinline__ Acc acc_add(Acc a, const Acc &b) { ring_add<L>(a, b); return a; }
+    static __device__ __forceinline__ Acc acc_norm(const Acc &a) { return a; }
     static __device__ __forceinline__ Acc shfl_down(const Acc &a, int d) {
         Acc r;
 #pragma unroll
@@ -888,29 +900,6 @@ __device__ __forceinline__ void elim_tasks(const WalkArgs &wa) {
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
         if (lane == 0) A::acc_store(wa.task_out + task * (u64)A::ACC_WORDS, acc);
-    }
-}
-
-// ------------------------------------------------------------------ final reduction
-// One block sums the task results in a fixed order (deterministic).
-
-template <class A>
-__device__ __forceinline__ void reduce_tasks(const u64 *task_out, u64 ntasks, u64 *result) {
-    __shared__ u64 sh[32 * 6];
-    typename A::Acc acc = A::acc_zero();
-    for (u64 t = threadIdx.x; t < ntasks; t += blockDim.x)
-        acc = A::acc_add(acc, A::acc_load(task_out + t * (u64)A::ACC_WORDS));
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) A::acc_store(sh + warp * A::ACC_WORDS, acc);
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        acc = lane < nw ? A::acc_load(sh + lane * A::ACC_WORDS) : A::acc_zero();
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
-        if (lane == 0) A::acc_store(result, acc);
     }
 }
 

@@ -1,5 +1,7 @@
 // generic.cu -- dispatch to the precompiled generic kernels, and the final
 // reduction kernels.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "core.cuh"
@@ -7,9 +9,60 @@
 
 namespace pk {
 
+// ------------------------------------------------------------------ final reduction
+// Task results summed in a fixed order (deterministic): block b takes tasks
+// [b per, (b + 1) per), and the last block to finish adds the blocks' sums in
+// block order.  A block's sum takes the place of its first task's result.
+// (FP64 runs at 2 lanes per clock and SM, so one block of 1024 threads spent
+// 25-38 us in its shuffle trees; blocks of 128 threads over the whole GPU
+// spend a few.)
 template <class A>
-__global__ void __launch_bounds__(1024) k_reduce(const u64 *task_out, u64 ntasks, u64 *result) {
-    reduce_tasks<A>(task_out, ntasks, result);
+__device__ __forceinline__ typename A::Acc block_sum(typename A::Acc acc, u64 *sh) {
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    if (lane == 0) A::acc_store(sh + warp * A::ACC_WORDS, acc);
+    __syncthreads();
+    acc = A::acc_load(sh);
+    for (int w = 1; w < nw; ++w) acc = A::acc_add(acc, A::acc_load(sh + w * A::ACC_WORDS));
+    return acc;   // (in every thread)
+}
+
+template <class A>
+__device__ __forceinline__ void reduce_tasks(u64 *task_out, u64 ntasks, u64 per, u64 *result, u64 *done_blocks) {
+    __shared__ u64 sh[32 * 6];
+    __shared__ int last;
+    typename A::Acc acc = A::acc_zero();
+    const u64 b = blockIdx.x * per, e = b + per < ntasks ? b + per : ntasks;
+    for (u64 t = b + threadIdx.x; t < e; t += blockDim.x)
+        acc = A::acc_add(acc, A::acc_load(task_out + t * (u64)A::ACC_WORDS));
+    acc = block_sum<A>(acc, sh);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) A::acc_store(result, A::acc_norm(acc));
+        return;
+    }
+    if (threadIdx.x == 0) {
+        A::acc_store(task_out + b * (u64)A::ACC_WORDS, acc);
+        __threadfence();
+        last = atomicAdd(done_blocks, 1ull) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    acc = A::acc_zero();
+    for (u64 k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
+        u64 w[A::ACC_WORDS];
+#pragma unroll
+        for (int i = 0; i < A::ACC_WORDS; ++i) w[i] = ((volatile u64 *)task_out)[k * per * (u64)A::ACC_WORDS + i];
+        acc = A::acc_add(acc, A::acc_load(w));
+    }
+    acc = block_sum<A>(acc, sh);
+    if (threadIdx.x == 0) A::acc_store(result, A::acc_norm(acc));
+}
+
+template <class A>
+__global__ void __launch_bounds__(128) k_reduce(u64 *task_out, u64 ntasks, u64 per, u64 *result, u64 *done_blocks) {
+    reduce_tasks<A>(task_out, ntasks, per, result, done_blocks);
 }
 
 // One warp per matrix, lane-strided then a fixed shuffle tree: deterministic.
@@ -25,7 +78,7 @@ __global__ void __launch_bounds__(256) k_batch_reduce(const BatchMat *mats, int 
     for (u64 t = b + lane; t < e; t += 32) acc = A::acc_add(acc, A::acc_load(task_out + t * (u64)A::ACC_WORDS));
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
-    if (lane == 0) A::acc_store(result + (u64)m * A::ACC_WORDS, acc);
+    if (lane == 0) A::acc_store(result + (u64)m * A::ACC_WORDS, A::acc_norm(acc));
 }
 
 // Serving: segment m sums pool[seg[2m] .. seg[2m] + seg[2m+1]) (task units),
@@ -40,7 +93,7 @@ __global__ void __launch_bounds__(256) k_segment_reduce(const u64 *seg, int nseg
     for (u64 t = b + lane; t < e; t += 32) acc = A::acc_add(acc, A::acc_load(pool + t * (u64)A::ACC_WORDS));
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
-    if (lane == 0) A::acc_store(result + (u64)m * 4, acc);
+    if (lane == 0) A::acc_store(result + (u64)m * 4, A::acc_norm(acc));
 }
 
 }  // namespace pk
@@ -101,14 +154,19 @@ GenericFns generic_fns(int nmax, int kind) {
     }
 }
 
-cudaError_t reduce_launch(int arith, const uint64_t *task_out, uint64_t ntasks, uint64_t *result, cudaStream_t st) {
-    const unsigned long long *in = reinterpret_cast<const unsigned long long *>(task_out);
+cudaError_t reduce_launch(int arith, uint64_t *task_out, uint64_t ntasks, uint64_t *result, uint64_t *done_blocks,
+                          cudaStream_t st) {
+    unsigned long long *in = reinterpret_cast<unsigned long long *>(task_out);
     unsigned long long *out = reinterpret_cast<unsigned long long *>(result);
+    unsigned long long *dn = reinterpret_cast<unsigned long long *>(done_blocks);
+    // 512 tasks a block (four additions a thread) until the GPU is full
+    const unsigned long long per = std::max<unsigned long long>(512, (ntasks + 151) / 152);
+    const unsigned grid = (unsigned)std::max<unsigned long long>(1, (ntasks + per - 1) / per);
     switch (arith) {
-    case 0: pk::k_reduce<pk::ArithF64><<<1, 1024, 0, st>>>(in, ntasks, out); break;
-    case 1: pk::k_reduce<pk::ArithExact<2>><<<1, 1024, 0, st>>>(in, ntasks, out); break;
-    case 2: pk::k_reduce<pk::ArithExact<4>><<<1, 1024, 0, st>>>(in, ntasks, out); break;
-    case 3: pk::k_reduce<pk::ArithExact<6>><<<1, 1024, 0, st>>>(in, ntasks, out); break;
+    case 0: pk::k_reduce<pk::ArithF64><<<grid, 128, 0, st>>>(in, ntasks, per, out, dn); break;
+    case 1: pk::k_reduce<pk::ArithExact<2>><<<grid, 128, 0, st>>>(in, ntasks, per, out, dn); break;
+    case 2: pk::k_reduce<pk::ArithExact<4>><<<grid, 128, 0, st>>>(in, ntasks, per, out, dn); break;
+    case 3: pk::k_reduce<pk::ArithExact<6>><<<grid, 128, 0, st>>>(in, ntasks, per, out, dn); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

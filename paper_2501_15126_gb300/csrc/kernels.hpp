@@ -44,8 +44,9 @@ cudaError_t xshared_launch(const pk::WalkArgs &wa, const void *img, int img_byte
                            int block, cudaStream_t st);
 cudaError_t xshared_attr(cudaFuncAttributes *attr);
 
-// Sums ntasks task results (words per task: 2 for FP64, arith for exact) in a
-// fixed order into result.
-cudaError_t reduce_launch(int arith, const uint64_t *task_out, uint64_t ntasks, uint64_t *result, cudaStream_t st);
+// Sums ntasks task results (words per task: 3 for FP64, arith for exact) in a
+// fixed order into result; task_out is overwritten, *done_blocks starts at 0.
+cudaError_t reduce_launch(int arith, uint64_t *task_out, uint64_t ntasks, uint64_t *result, uint64_t *done_blocks,
+                          cudaStream_t st);
 
 }  // namespace perm

@@ -30,7 +30,7 @@ namespace {
 
 constexpr size_t kNoAllocScratchBytes = 1u << 20;
 constexpr int kNoAllocMaxN = 48;                  // the generic kernels' largest bucket
-constexpr size_t kOffCounters = 0;                // [0] task counter, [1] skipped blocks, [2] deadline, [3] abort
+constexpr size_t kOffCounters = 0;                // [0] task counter, [1] skipped blocks, [2] deadline, [3] abort, [4] reduction
 constexpr size_t kOffResult = 128;                // up to 3 words
 constexpr size_t kOffBatchMat = 192;              // one pk::BatchMat
 constexpr size_t kOffImage = 256;                 // the matrix image (<= 20480 bytes)
@@ -158,7 +158,7 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
         ba.abort_flag = reinterpret_cast<unsigned int *>(d_counters + 3);
         if ((e = P.gf.walk(ba, P.grid, P.block, st_)) != cudaSuccess) return failed(cuda_fail(e, "walk kernel launch"));
     }
-    if ((e = reduce_launch(P.arith, reinterpret_cast<const uint64_t *>(d_tasks), P.ntasks, d_result, st_)) !=
+    if ((e = reduce_launch(P.arith, reinterpret_cast<uint64_t *>(d_tasks), P.ntasks, d_result, d_counters + 4, st_)) !=
         cudaSuccess)
         return failed(cuda_fail(e, "reduce kernel launch"));
     uint64_t host[4];

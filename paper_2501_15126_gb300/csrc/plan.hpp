@@ -98,11 +98,13 @@ struct perm_plan_s {
 namespace perm {
 
 // Workspace layout (64-bit words): [0] task counter, [1] skipped blocks,
-// [2..4] reduced result, [5] deadline, [6] abort flag, [8..13] the
+// [2..4] reduced result, [5] deadline, [6] abort flag, [7] blocks of the
+// reduction that are done, [8..13] the
 // single-matrix BatchMat, [16..] task results.  Words 0..7 are cleared
 // before every launch.
 constexpr size_t kWsDeadline = 5;
 constexpr size_t kWsAbort = 6;
+constexpr size_t kWsReduced = 7;
 constexpr size_t kWsBatchMat = 8;
 constexpr size_t kWsTaskOut = 16;
 
