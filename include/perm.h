@@ -402,6 +402,19 @@ perm_status_t perm_codegen_source(const perm_matrix_t *A, const perm_opts_t *opt
 perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap,
                                int64_t *len, int32_t *k, int32_t *order);
 
+/* The program image that the precompiled eliminated walk reads for A (for
+   inspection): the same walk as perm_elim_source's, its step written as bundles
+   of four operations on numbered slots (start values, entries, flip lists of
+   the outer columns, program).  shared_launch = 1 plans as perm_batch and the
+   server do, 0 as a plan of its own.  *kind is the arithmetic (0 FP64, 1
+   double-double, else 2 limbs), the walk's sum is the true one times 2^-scale
+   and its sum of |terms| times 2^-abs_shift; *len is 0 where the chained walk
+   runs instead (n <= 8, n > 48, options as for perm_elim_source, or where the
+   chain counts fewer operations). */
+perm_status_t perm_elim_image(const perm_matrix_t *A, const perm_opts_t *opts, int32_t shared_launch, void *buf,
+                              int64_t cap, int64_t *len, int32_t *kind, int32_t *k, int32_t *order, int32_t *scale,
+                              int32_t *abs_shift);
+
 /* The matrix image that the precompiled generic kernels read for A (for
    inspection).  Sec. III names the sparse A and x as the two data
    structures the walk touches; this is A as those kernels keep it in

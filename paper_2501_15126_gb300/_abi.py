@@ -111,6 +111,8 @@ SIGNATURES = [
                                     ctypes.POINTER(c_i64)]),
     ("perm_elim_source", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), ctypes.c_char_p, c_i64,
                                  ctypes.POINTER(c_i64), ctypes.POINTER(c_i32), ctypes.POINTER(c_i32)]),
+    ("perm_elim_image", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), c_i32, c_vp, c_i64, ctypes.POINTER(c_i64)]
+     + [ctypes.POINTER(c_i32)] * 5),
     ("perm_generic_image", c_i32, [ctypes.POINTER(Matrix), ctypes.POINTER(Opts), c_vp, c_i64, ctypes.POINTER(c_i64),
                                    ctypes.POINTER(c_i32), ctypes.POINTER(c_i32), ctypes.POINTER(c_i32)]),
     ("perm_status_string", ctypes.c_char_p, [c_i32]),
@@ -285,6 +287,20 @@ def elim_source(a, **kw):
     check(lib().perm_elim_source(ctypes.byref(m.c), ctypes.byref(o), buf, n.value + 1, ctypes.byref(n), None, None),
           "perm_elim_source")
     return buf.value.decode(), k.value, list(order)[: m.c.n]
+
+
+def elim_image(a, shared_launch=False, **kw):
+    """perm_elim_image: (image bytes, kind, k, columns: outer by Gray position, low, last, scale, abs_shift)."""
+    m = a if isinstance(a, CSRMatrix) else CSRMatrix(a)
+    o = opts(**kw)
+    n, kind, k, order, scale, shift = c_i64(), c_i32(), c_i32(), (c_i32 * 64)(), c_i32(), c_i32()
+    args = [ctypes.byref(x) for x in (kind, k)] + [order] + [ctypes.byref(x) for x in (scale, shift)]
+    check(lib().perm_elim_image(ctypes.byref(m.c), ctypes.byref(o), int(shared_launch), None, 0, ctypes.byref(n), *args),
+          "perm_elim_image")
+    buf = ctypes.create_string_buffer(max(n.value, 1))
+    check(lib().perm_elim_image(ctypes.byref(m.c), ctypes.byref(o), int(shared_launch), buf, n.value, ctypes.byref(n), *args),
+          "perm_elim_image")
+    return buf.raw[: n.value], kind.value, k.value, list(order)[: m.c.n], scale.value, shift.value
 
 
 def generic_image(a, **kw):

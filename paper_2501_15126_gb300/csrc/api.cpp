@@ -95,7 +95,7 @@ void build_devmat(const Matrix &m, const Layout &L, int img, int nmax, std::vect
 // x0_i = a_{i,last} - (1/2) sum_j a_ij as an exact double-double (hi, lo):
 // halving is exact and every partial sum is accumulated with TwoSum, so no bit
 // is lost while the value fits 106 bits (values on a common 2^-53 grid do).
-static void x0_dd(const Matrix &m, int r, int last, double *hi_out, double *lo_out) {
+void x0_dd(const Matrix &m, int r, int last, double *hi_out, double *lo_out) {
     double hi = 0.0, lo = 0.0;
     auto add = [&](double v) {
         const double s = hi + v;
@@ -467,11 +467,70 @@ void codegen_choose_elim(perm_plan_s &P, int max_width) {
     P.use_elim = true;
 }
 
+// The precompiled eliminated walk of a plan that the generic engine runs.
+bool vm_rebuild(perm_plan_s &P) {
+    const int img = P.dd ? kImgDD : (P.m.is_int ? kImgInt : kImgF64);
+    const int limbs = P.m.is_int ? P.limbs : 0;
+    P.vm_img.clear();
+    if (!vm_image(P.m, P.elim, img, limbs, kVmMaxSlotsPerLane, P.vm_img)) return false;
+    const pk::VmHeader *H = reinterpret_cast<const pk::VmHeader *>(P.vm_img.data());
+    P.vm_bytes = P.vm_img.size() + vm_slot_area(img, limbs, H->nslots, H->nextra);
+    return P.vm_bytes <= (size_t)kVmMaxWarpBytes;
+}
+
+bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
+    P.vm = P.use_elim = false;
+    adopt_elim(P);
+    const int n = P.m.n;
+    if (!elim_allowed(P) || n < min_n || n > 48 || P.opts.engine == PERM_ENGINE_CODEGEN) return false;
+    const double range = std::log2((double)(P.g_hi - P.g_lo));
+    // Where the line lies: chained -> eliminated, single matrices: n=17 p=0.3 FP64
+    // 0.228 -> 0.024 ms, n=24 p=0.2 FP64 0.21 -> 0.039 ms and 0/1 0.082 -> 0.020 ms,
+    // n=28 p=0.3 FP64 3.0 -> 1.33 ms, n=23 p=0.25 double-double 0.95 -> 0.13 ms a
+    // call; n=28 p=0.4 0/1, whose rows share too much, stays with the chain (2.2 ms).
+    // The chained walk's time in lane-operations of the whole GPU.  Alone, a walk
+    // of fewer than 152 blocks' tasks (eight 32-chunk tasks of 2^8 steps, exact
+    // 2^6) leaves SMs idle; an exact chained step is about 90 instructions, an
+    // interpreted operation about 20.
+    const bool alone = full_blocks == kVmFullBlocks;
+    const double ops = P.m.is_int ? 90.0 : n > 32 ? cost_per_step(P.L, false) : cost_per_step_dual(P.L, true);
+    const double sms = alone ? std::min(152.0, std::max(1.0, std::exp2(range - (P.m.is_int ? 14.0 : 16.0)))) : 152.0;
+    const double chain = ops * std::exp2(range) * 152.0 / sms;
+    ElimLimits lim;
+    lim.full_blocks = full_blocks;
+    lim.allow_none = lim.tables_only = true;
+    lim.candidates = n <= 20 ? 4 : n <= 23 ? 8 : n <= 26 ? 16 : kNMax;
+    for (int width = 5; width >= 3; --width) {
+        lim.max_width = width;
+        if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;
+        const double steps = std::max(std::exp2(range - P.elim.k), full_blocks);
+        if ((P.elim.table_ops + 10.0) * (P.m.is_int ? 20.0 : 1.0) * steps > 0.9 * chain) return false;
+        P.vm = P.use_elim = true;
+        if (vm_rebuild(P)) {
+            adopt_elim(P);
+            return true;
+        }
+        P.vm = P.use_elim = false;
+        P.vm_img.clear();
+    }
+    return false;
+}
+
+void choose_shared_chunks(perm_plan_s &P, int max_tasks_log2) {
+    const int h = P.elim.h;
+    int K = std::max(0, std::min(3, h - 5));   // 2^3 outer steps a lane, and full warps first
+    K = std::max(K, h - 5 - max_tasks_log2);
+    P.K = K;
+    P.chunk_lo = 0;
+    P.chunk_hi = 1ull << (h - K);
+    P.ntasks = (P.chunk_hi + 31) / 32;
+}
+
 // Switches a plan to (or from) the scales of the eliminated walk's sums.
 void adopt_elim(perm_plan_s &P) {
     P.val_shift = P.use_elim ? P.elim.scale : 0;
     if (!P.m.is_int)
-        P.abs_shift = P.use_elim ? P.elim.scale - P.m.n * elim_abs_bits(P.m.n, P.elim.k) : abs_shift_for(P.m);
+        P.abs_shift = P.use_elim ? P.elim.scale : abs_shift_for(P.m);
     if (!P.use_elim) return;
     P.k = P.m.n;
     P.c = P.m.n - 1;
@@ -513,6 +572,19 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
         if ((e = xshared_occupancy(n, (int)P.img_bytes, 256, &bps)) != cudaSuccess) return cuda_fail(e, "occupancy");
         perm_status_t st = choose_launch(P, 0, std::max(bps, 1), 256);
         if (st != PERM_OK) return st;
+    } else if (engine == PERM_ENGINE_GENERIC && !tiny && vm_prepare(P, kVmFullBlocks, 9)) {
+        P.gf = generic_fns(P.family_nmax(), P.family_kind());
+        if (!P.gf.walk) return fail(PERM_ERR_INTERNAL, "no eliminated walk for this arithmetic");
+        P.img_bytes = P.vm_bytes;
+        if ((e = cudaMalloc(&P.d_devmat, P.vm_img.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc(program image)");
+        if ((e = cudaMemcpy(P.d_devmat, P.vm_img.data(), P.vm_img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+            return cuda_fail(e, "cudaMemcpy(program image)");
+        cudaFuncAttributes attr;
+        if ((e = P.gf.attr(&attr)) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
+        P.regs = attr.numRegs;
+        int bps = 0;
+        if ((e = P.gf.occ(32, P.vm_bytes, &bps)) != cudaSuccess) return cuda_fail(e, "occupancy");
+        choose_launch_elim(P, std::max(bps, 1), 32);
     } else if (engine == PERM_ENGINE_GENERIC) {
         P.gf = generic_fns(nmax, P.kind());
         if (!P.gf.walk) return fail(PERM_ERR_INTERNAL, "no generic kernel for this size");
@@ -826,6 +898,13 @@ static perm_status_t make_dd_plan(perm_plan_s &P) {
 
 }  // namespace perm
 
+// Shared-memory classes of the eliminated walk: a launch takes the largest
+// program's region for every warp, so small programs keep to themselves.
+int perm_plan_s::family_nmax() const {
+    if (!vm) return perm::nmax_bucket(m.n);
+    return vm_bytes <= 20 * 1024 ? 1 : vm_bytes <= 44 * 1024 ? 2 : 3;
+}
+
 perm_plan_s::~perm_plan_s() {
     if (d_devmat) cudaFree(d_devmat);
     if (d_ws) cudaFree(d_ws);
@@ -995,6 +1074,33 @@ perm_status_t perm_codegen_source(const perm_matrix_t *A, const perm_opts_t *opt
     return PERM_OK;
 }
 
+// The outer columns by Gray position, the low columns, the last column.
+static void elim_order(const perm_plan_s &P, int32_t *order) {
+    if (!order) return;
+    for (int i = 0; i < P.m.n; ++i)
+        order[i] = !P.use_elim ? P.L.col_order[i]
+                   : i < P.elim.h ? P.elim.outer[i]
+                   : i < P.m.n - 1 ? P.elim.low[i - P.elim.h]
+                                   : P.elim.last;
+}
+
+perm_status_t perm_elim_image(const perm_matrix_t *A, const perm_opts_t *opts, int32_t shared_launch, void *buf,
+                              int64_t cap, int64_t *len, int32_t *kind, int32_t *k, int32_t *order, int32_t *scale,
+                              int32_t *abs_shift) {
+    perm_plan_s P;
+    perm_status_t st = plan_prepare(A, opts, P);
+    if (st != PERM_OK) return st;
+    if (P.m.n > 8 && P.m.n <= 48) vm_prepare(P, shared_launch ? kVmFullBlocksShared : kVmFullBlocks, 9);
+    if (len) *len = (int64_t)P.vm_img.size();
+    if (kind) *kind = P.family_kind();
+    if (k) *k = P.vm ? P.elim.k : 0;
+    if (scale) *scale = P.val_shift;
+    if (abs_shift) *abs_shift = P.abs_shift;
+    elim_order(P, order);
+    if (buf && cap > 0) std::memcpy(buf, P.vm_img.data(), std::min<size_t>((size_t)cap, P.vm_img.size()));
+    return PERM_OK;
+}
+
 perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap, int64_t *len,
                                int32_t *k, int32_t *outer) {
     perm_plan_s P;
@@ -1005,12 +1111,7 @@ perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, 
     std::string src = P.use_elim ? elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs) : std::string();
     adopt_elim(P);
     if (k) *k = P.use_elim ? P.elim.k : 0;
-    if (outer)   // the outer columns by Gray position, the low columns, the last column
-        for (int i = 0; i < P.m.n; ++i)
-            outer[i] = !P.use_elim ? P.L.col_order[i]
-                       : i < P.elim.h ? P.elim.outer[i]
-                       : i < P.m.n - 1 ? P.elim.low[i - P.elim.h]
-                                       : P.elim.last;
+    elim_order(P, outer);
     if (len) *len = (int64_t)src.size();
     if (buf && cap > 0) {
         const size_t nb = std::min<size_t>((size_t)cap - 1, src.size());

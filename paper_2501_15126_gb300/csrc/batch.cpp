@@ -51,11 +51,14 @@ int BatchGroup::setup(int nmax_, int kind_, int K_target) {
     ntasks = 0;
     for (size_t i = 0; i < plans.size(); ++i) {
         perm_plan_s &P = *plans[i];
-        const int K = batch_chunk_log2(P.m.n, gf.block_log2, K_target);
-        P.K = K;
-        P.chunk_lo = 0;
-        P.chunk_hi = P.total >> K;
-        P.ntasks = (P.chunk_hi + 31) / 32;
+        if (P.vm) {
+            choose_shared_chunks(P, 26);
+        } else {
+            P.K = batch_chunk_log2(P.m.n, gf.block_log2, K_target);
+            P.chunk_lo = 0;
+            P.chunk_hi = P.total >> P.K;
+            P.ntasks = (P.chunk_hi + 31) / 32;
+        }
         P.engine = PERM_ENGINE_GENERIC;
         P.gf = gf;
         P.nmax = nmax;
@@ -64,7 +67,7 @@ int BatchGroup::setup(int nmax_, int kind_, int K_target) {
         mats[i].chunk_lo = 0;
         mats[i].chunk_hi = P.chunk_hi;
         mats[i].out_offset = ntasks;
-        mats[i].K = K;
+        mats[i].K = P.K;
         mats[i].abs_shift = P.abs_shift;
         ntasks += P.ntasks;
     }
@@ -72,20 +75,24 @@ int BatchGroup::setup(int nmax_, int kind_, int K_target) {
     size_t total = 0;
     slot_bytes = 16;
     for (size_t i = 0; i < plans.size(); ++i) {
-        const size_t b = devmat_bytes_for(plans[i]->L, img, nmax);
+        const perm_plan_s &P = *plans[i];
+        const size_t b = P.vm ? P.vm_img.size() : devmat_bytes_for(P.L, img, nmax);
         mats[i].image = (int)(total / 16);
         total += b;
-        slot_bytes = std::max(slot_bytes, b);
+        slot_bytes = std::max(slot_bytes, P.vm ? P.vm_bytes : b);
     }
     images.assign(total, 0);
-    for (size_t i = 0; i < plans.size(); ++i)
-        build_devmat_into(plans[i]->m, plans[i]->L, img, nmax, images.data() + (size_t)mats[i].image * 16);
+    for (size_t i = 0; i < plans.size(); ++i) {
+        unsigned char *dst = images.data() + (size_t)mats[i].image * 16;
+        if (plans[i]->vm) std::memcpy(dst, plans[i]->vm_img.data(), plans[i]->vm_img.size());
+        else build_devmat_into(plans[i]->m, plans[i]->L, img, nmax, dst);
+    }
     cudaFuncAttributes attr;
     if (gf.attr(&attr) == cudaSuccess) regs = attr.numRegs;
     int bps = 0;
-    cudaError_t e = gf.occ(256, slot_bytes, &bps);
+    block = nmax < 16 ? 32 : 256;   // the eliminated walk runs one warp per block
+    cudaError_t e = gf.occ(block, slot_bytes, &bps);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy");
-    block = 256;
     int64_t g = (int64_t)kSMCount * std::max(bps, 1);
     g = std::min<int64_t>(g, ((int64_t)ntasks * 32 + block - 1) / block);
     grid = (int)std::max<int64_t>(1, g);
@@ -205,7 +212,7 @@ static perm_status_t run_groups(std::map<std::pair<int, int>, BatchGroup> &group
         BatchGroup &G = kv.second;
         G.timeout_ns = (unsigned long long)std::max(0, opts.timeout_ms) * 1000000ull;
         int K_target = opts.chunk_log2;
-        if (!K_target) {
+        if (!K_target && kv.first.first >= 16) {
             if (!chunk_log2_is_tuned(kv.first.first, kv.first.second)) {
                 G.nmax = kv.first.first;
                 G.kind = kv.first.second;
@@ -332,6 +339,7 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
             for (int32_t i = t; i < count; i += nthreads) {
                 plans[i].reset(new perm_plan_s());
                 prep[i] = plan_prepare(&mats[i], &opts, *plans[i]);
+                if (prep[i] == PERM_OK && !plans[i]->zero) vm_prepare(*plans[i], kVmFullBlocksShared, kVmMinBatch);
             }
         };
         std::vector<std::thread> pool;
@@ -353,7 +361,7 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
         }
         if (P.zero) { describe(P, &out[i]); out[i].status = PERM_OK; plans[i].reset(); continue; }
         if (P.m.n <= 8 || P.m.n > 48) { singles.push_back(i); continue; }
-        groups[{nmax_bucket(P.m.n), P.kind()}].add(i, &P);
+        groups[{P.family_nmax(), P.family_kind()}].add(i, &P);
     }
     const double t_prep = now_ms() - t0;
     if (opts.timeout_ms < 0) return fail(PERM_ERR_ARG, "timeout_ms < 0");
@@ -371,7 +379,11 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
             if (!P.m.is_int && !P.dd && opts.precision == PERM_PREC_AUTO && P.m.n <= kAutoDDMaxN &&
                 out[i].status == PERM_OK && needs_dd(P.m.n, out[i].f64 + out[i].f64_lo, out[i].abs_term_sum)) {
                 P.dd = true;
-                redo[{nmax_bucket(P.m.n), P.kind()}].add(i, &P);
+                if (P.vm && !vm_rebuild(P)) {   // too many pair slots: the chained walk
+                    P.vm = P.use_elim = false;
+                    adopt_elim(P);
+                }
+                redo[{P.family_nmax(), P.family_kind()}].add(i, &P);
             }
         }
     if (!redo.empty()) {

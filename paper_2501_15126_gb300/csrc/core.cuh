@@ -121,6 +121,15 @@ __device__ __forceinline__ float abs_scaled_f32(double t, int shift) {
     return __int_as_float(h << 3);
 }
 
+// The same, unscaled, with the top 23 fraction bits (relative error below
+// 2^-23): the eliminated walk multiplies the magnitudes of up to 64 rows, whose
+// errors add up (with 20 bits each, 1e-5 at n = 28).  Its values are below 2^121
+// (elim_row_bits), so only the small end is clamped.
+__device__ __forceinline__ float abs_f32_full(double t) {
+    const int h = max((__double2hiint(t) & 0x7fffffff) - 896 * (1 << 20), 0);
+    return __int_as_float((h << 3) | (int)((u32)__double2loint(t) >> 29));
+}
+
 // ------------------------------------------------------------------ FP64 arithmetic
 
 struct ArithF64 {

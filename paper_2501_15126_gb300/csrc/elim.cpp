@@ -18,7 +18,6 @@ inline int pc(uint64_t v) { return __builtin_popcountll(v); }
 // is fused with the subtraction of the column-on half.
 struct Sim {
     double ops = 0.0;
-    int width = 0;
     int order[kNMax];
 };
 
@@ -41,55 +40,60 @@ int bucket_order(const uint64_t *scope, const int *idx, int t, int *seq) {
     return pc(u);
 }
 
-void simulate(const uint64_t *rowmask, int n, uint64_t L, int max_width, Sim &S) {
-    uint64_t tabs[2 * kNMax];
+// (The column graph is enough to pick the next column: adj[c] is the joint scope
+// of the tables that mention c.  `cap` gives up once the count passes it.)
+void simulate(const uint64_t *rowmask, int n, uint64_t L, int max_width, double cap, Sim &S) {
+    uint64_t tabs[2 * kNMax], adj[kNMax];
     int nt = 0, scalars = 0;
-    S.ops = 0.0;
-    S.width = 0;
+    double ops = 0.0;
+    S.ops = 1e30;
+    for (uint64_t x = L; x; x &= x - 1) adj[__builtin_ctzll(x)] = 0;
     for (int i = 0; i < n; ++i) {
         const uint64_t s = rowmask[i] & L;
         if (!s) { ++scalars; continue; }
-        S.ops += (double)(1ull << pc(s)) - 1.0;
+        const int w = pc(s);
+        if (w > max_width) return;
+        ops += (double)((1u << w) - 1u);
         tabs[nt++] = s;
-        S.width = std::max(S.width, pc(s));
+        for (uint64_t x = s; x; x &= x - 1) adj[__builtin_ctzll(x)] |= s;
     }
-    if (S.width > max_width) { S.ops = 1e30; return; }
     uint64_t rem = L;
     int done = 0;
     while (rem) {
-        int bw = 1 << 30;
-        uint64_t bb = 0;
+        int c = -1, bw = 1 << 30;
         for (uint64_t x = rem; x; x &= x - 1) {
-            const uint64_t b = x & (~x + 1);
-            uint64_t u = 0;
-            int cnt = 0;
-            for (int t = 0; t < nt; ++t)
-                if (tabs[t] & b) { u |= tabs[t]; ++cnt; }
-            const int key = pc(u) * 256 + cnt;
-            if (key < bw) { bw = key; bb = b; }
+            const int j = __builtin_ctzll(x), w = pc(adj[j]);
+            if (w < bw) { bw = w; c = j; }
         }
-        int idx[2 * kNMax], seq[2 * kNMax], t = 0;
-        for (int i = 0; i < nt; ++i)
-            if (tabs[i] & bb) idx[t++] = i;
-        const int w = bucket_order(tabs, idx, t, seq);
-        S.width = std::max(S.width, w);
-        if (w > max_width) { S.ops = 1e30; return; }
-        uint64_t u = tabs[seq[0]];
-        if (t == 1) S.ops += std::ldexp(1.0, pc(u) - 1);
-        for (int i = 1; i < t; ++i) {
-            u |= tabs[seq[i]];
-            S.ops += std::ldexp(1.0, pc(u));
+        if (bw > max_width) return;
+        const uint64_t b = 1ull << c;
+        // the bucket's tables by scope size: multiplied smallest first
+        uint64_t bucket[2 * kNMax];
+        int t = 0, keep = 0;
+        for (int i = 0; i < nt; ++i) {
+            if (!(tabs[i] & b)) { tabs[keep++] = tabs[i]; continue; }
+            int p = t++;
+            for (; p > 0 && pc(bucket[p - 1]) > pc(tabs[i]); --p) bucket[p] = bucket[p - 1];
+            bucket[p] = tabs[i];
         }
-        int keep = 0;
-        for (int i = 0; i < nt; ++i)
-            if (!(tabs[i] & bb)) tabs[keep++] = tabs[i];
         nt = keep;
-        u &= ~bb;
+        uint64_t u = bucket[0];
+        if (t == 1) ops += 0.5 * (double)(1u << pc(u));
+        for (int i = 1; i < t; ++i) {
+            u |= bucket[i];
+            ops += (double)(1u << pc(u));
+        }
+        if (ops > cap) return;
+        u &= ~b;
         if (u) tabs[nt++] = u; else ++scalars;
-        S.order[done++] = __builtin_ctzll(bb);
-        rem &= ~bb;
+        for (uint64_t x = u; x; x &= x - 1) {
+            const int j = __builtin_ctzll(x);
+            adj[j] = (adj[j] | u) & ~b;
+        }
+        S.order[done++] = c;
+        rem &= ~b;
     }
-    S.ops += std::max(0, scalars - 1);
+    S.ops = ops + std::max(0, scalars - 1);
 }
 
 // Compresses the bits of `v` selected by `mask` (software pext; n <= 64).
@@ -224,11 +228,109 @@ struct Builder {
         // the scalars' product (exact: smallest bounds first, so that the
         // factors stay in 32 bits as long as they can)
         if (exact) std::stable_sort(scalars.begin(), scalars.end(), [&](int a, int b) { return E.bound[a] < E.bound[b]; });
+        // (FP64: pairwise, so that the last products do not wait on one another)
+        if (!exact)
+            while (scalars.size() > 2) {
+                std::vector<int> half;
+                for (size_t i = 0; i + 1 < scalars.size(); i += 2) half.push_back(mul(scalars[i], scalars[i + 1]));
+                if (scalars.size() & 1) half.push_back(scalars.back());
+                scalars = half;
+            }
         int r = scalars[0];
         for (size_t i = 1; i < scalars.size(); ++i) r = mul(r, scalars[i]);
         E.result = r;
     }
 };
+
+// The program by tables (scopes in elimination-order bits).
+void build_tables(const Matrix &m, ElimPlan &E, const int *order, int k) {
+    const int n = m.n;
+    E.tables.clear();
+    E.tops.clear();
+    E.factors.clear();
+    E.table_ops = 0.0;
+    uint64_t live[kNMax];   // scope of each row by elimination place
+    for (int i = 0; i < n; ++i) live[i] = 0;
+    for (int q = 0; q < k; ++q)
+        for (uint64_t rows = m.colmask[order[q]]; rows; rows &= rows - 1) live[__builtin_ctzll(rows)] |= 1ull << q;
+    int item_tab[2 * kNMax], nitems = 0;   // tables (or rows still to be made tables: -1 - row) by scope
+    uint64_t item_scope[2 * kNMax];
+    for (int i = 0; i < n; ++i) {
+        double b = 0.0;
+        if (m.is_int)
+            for (int j = 0; j < n; ++j) b += std::fabs(m.fval(i, j));
+        E.tables.push_back({0, std::max(b, 1.0), i});
+        if (live[i]) {
+            item_scope[nitems] = live[i];
+            item_tab[nitems++] = -1 - i;
+        } else {
+            E.factors.push_back(i);
+        }
+    }
+    auto make = [&](uint64_t scope, double bound) {
+        E.tables.push_back({scope, bound, -1});
+        return (int)E.tables.size() - 1;
+    };
+    for (int q = 0; q < k; ++q) {
+        const uint64_t b = 1ull << q;
+        int idx[2 * kNMax], seq[2 * kNMax], t = 0;
+        for (int i = 0; i < nitems; ++i)
+            if (item_scope[i] & b) idx[t++] = i;
+        if (!t) continue;
+        bucket_order(item_scope, idx, t, seq);
+        // a row becomes a table just before it is multiplied, and up to three more of
+        // the bucket's rows of the same small size with it (one instruction)
+        auto make_row = [&](int it) {
+            const int row = -1 - item_tab[it];
+            item_tab[it] = make(item_scope[it], E.tables[row].bound);
+            E.tops.push_back({kTabRow, item_tab[it], row, 0, 0});
+            E.table_ops += (double)(1ull << pc(item_scope[it])) - 1.0;
+        };
+        auto table = [&](int at) {
+            const int it = seq[at];
+            if (item_tab[it] >= 0) return item_tab[it];
+            make_row(it);
+            const int w = pc(item_scope[it]);
+            for (int s = at + 1, more = 3; s < t && more > 0 && w <= 3; ++s)
+                if (item_tab[seq[s]] < 0 && pc(item_scope[seq[s]]) == w) { make_row(seq[s]); --more; }
+            return item_tab[it];
+        };
+        int cur = table(0), out;
+        uint64_t scope = item_scope[seq[0]];
+        if (t == 1) {
+            out = make(scope & ~b, 2.0 * E.tables[cur].bound);
+            E.tops.push_back({kTabSub, out, cur, cur, q});
+            E.table_ops += (double)(1ull << (pc(scope) - 1));
+        } else {
+            for (int s = 1; s < t; ++s) {
+                const int r = table(s);
+                scope |= item_scope[seq[s]];
+                const double bound = E.tables[cur].bound * E.tables[r].bound;
+                const bool last = s + 1 == t;
+                const int d = last ? make(scope & ~b, 2.0 * bound) : make(scope, bound);
+                E.tops.push_back({(uint8_t)(last ? kTabSum : kTabMul), d, cur, r, q});
+                E.table_ops += (double)(1ull << pc(scope));
+                cur = d;
+            }
+            out = cur;
+        }
+        int keep = 0;
+        for (int i = 0; i < nitems; ++i)
+            if (!(item_scope[i] & b)) {
+                item_scope[keep] = item_scope[i];
+                item_tab[keep++] = item_tab[i];
+            }
+        nitems = keep;
+        const uint64_t left = scope & ~b;
+        if (left) {
+            item_scope[nitems] = left;
+            item_tab[nitems++] = out;
+        } else {
+            E.factors.push_back(out);
+        }
+    }
+    E.table_ops += (double)E.factors.size() - 1.0;
+}
 
 }  // namespace
 
@@ -250,6 +352,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
     int k = 0;
     double best_time = 1e300;
     Sim best, S;
+    best.ops = n - 1;
     auto model = [&](double ops, int kk, uint64_t LL) {
         double flip = 0.0;
         int got = 0;
@@ -257,6 +360,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
             if (!((LL >> cand[i]) & 1ull)) { flip += pc(m.colmask[cand[i]]) * 0.75; ++got; }
         return (ops + flip + 8.0) * std::max(std::exp2(range_log2 - kk), lim.full_blocks);
     };
+    if (lim.allow_none) best_time = model(n - 1, 0, 0);
     for (;;) {
         int pick = -1;
         Sim pick_sim;
@@ -267,7 +371,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
             if ((L >> c) & 1ull) continue;
             ++tried;
             if (range_log2 - (k + 1) < 0.0) continue;
-            simulate(rows, n, L | (1ull << c), lim.max_width, S);
+            simulate(rows, n, L | (1ull << c), lim.max_width, lim.max_ops, S);
             if (S.ops > lim.max_ops) continue;
             const double t = model(S.ops, k + 1, L | (1ull << c));
             if (t < pick_time) { pick_time = t; pick = c; pick_sim = S; }
@@ -278,7 +382,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
         L |= 1ull << pick;
         ++k;
     }
-    if (k < 1) return false;
+    if (k < 1 && !lim.allow_none) return false;
     E.n = n;
     E.k = k;
     E.h = n - 1 - k;
@@ -298,12 +402,20 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
         for (int j = 0; j < n; ++j) rs += std::fabs(m.fval(i, j));
         if (!(rs > 0.0) || !std::isfinite(rs)) return false;
         std::frexp(rs / 2.0, &E.exp2[i]);
+        E.exp2[i] -= elim_row_bits(n, k);
         E.scale += E.exp2[i];
     }
-    Builder(m, E).run(L, E.low, k);
+    double count;
+    if (lim.tables_only) {
+        build_tables(m, E, E.low, k);
+        count = E.table_ops;
+    } else {
+        Builder(m, E).run(L, E.low, k);
+        count = (double)E.ops.size();
+    }
     double flips = 0.0;
     for (int p = 0; p < h; ++p) flips += pc(m.colmask[E.outer[p]]) * std::ldexp(1.0, -(p + 1));
-    E.ops_per_step = std::ldexp((double)E.ops.size() + flips + 1.0, -k);
+    E.ops_per_step = std::ldexp(count + flips + 1.0, -k);
     return true;
 }
 
@@ -332,9 +444,7 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
     else o << "typedef ArithExact<" << limbs << "> A;\n";
     o << "struct ElimPol {\n    static constexpr int NX = " << n << ";\n";
     o << "    static constexpr bool kAbs = " << (want_abs ? "true" : "false") << ";\n";
-    o << "    // the walk's sum is the true one times 2^-scale, its sum of |terms| times 2^-abs_shift\n";
-    o << "    static constexpr int scale = " << E.scale << ";\n";
-    o << "    static constexpr int abs_shift = " << E.scale - (fp ? n * elim_abs_bits(n, E.k) : 0) << ";\n";
+    o << "    static constexpr int scale = " << E.scale << ";   // the walk's sums are the true ones times 2^-scale\n";
     o << "    typedef A::X X;\n";
     auto entry = [&](int r, int c) {
         return fp ? dlit(std::ldexp(m.fval(r, c), -E.exp2[r])) : ilit(2 * m.ival(r, c));
@@ -372,7 +482,7 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
     static const char *const tn[3] = {"int", "i64", "Ring<A::L>"};
     o << "    static __device__ __forceinline__ void step(const X (&x)[NX], A::Blk &blk, bool odd) {\n";
     if (want_abs)
-        for (int i = 0; i < n; ++i) o << "        const float f" << i << " = abs_scaled_f32(x[" << i << "], kAbsRow);\n";
+        for (int i = 0; i < n; ++i) o << "        const float f" << i << " = abs_f32_full(x[" << i << "]);\n";
     for (size_t q = 0; q < E.ops.size(); ++q) {
         const ElimOp &op = E.ops[q];
         const int v = n + (int)q;
@@ -388,7 +498,7 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
             if (!want_abs) continue;
             o << "        const float f" << v << " = ";
             switch (op.kind) {
-            case kElimAdd: o << "abs_scaled_f32(v" << v << ", kAbsRow)"; break;
+            case kElimAdd: o << "abs_f32_full(v" << v << ")"; break;
             case kElimMul: o << "f" << op.a << " * f" << op.b; break;
             case kElimMulSub: o << "f" << op.a << " * f" << op.b << " + f" << op.c; break;
             default: o << "f" << op.a << " + f" << op.b; break;
@@ -435,7 +545,6 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
         o << "        if (odd) A::blk_add<-1>(blk, t); else A::blk_add<1>(blk, t);\n";
     }
     o << "    }\n";
-    if (want_abs) o << "    static constexpr int kAbsRow = " << -elim_abs_bits(n, E.k) << ";\n";
     o << "};\n}  // namespace pk\n\n";
     // One block per SM (255 registers): FP64 steps are bound by the FP64 pipe (2
     // lane-operations per clock and SM), which eight warps fill, and the tables

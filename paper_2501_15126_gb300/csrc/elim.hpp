@@ -38,16 +38,35 @@ struct ElimOp {
     int32_t a, b, c;
 };
 
+// The same program by whole tables (the precompiled kernels' form).  Tables are
+// numbered; entry e of a table belongs to the setting e of its scope's columns,
+// lowest bit the column summed out first.
+struct ElimTable {
+    uint64_t scope;    // bit q: the q-th column summed out (elimination order)
+    double bound;      // exact: a bound of every entry's magnitude
+    int row;           // >= 0: single value x_row (scope empty)
+};
+enum ElimTableKind : uint8_t { kTabRow = 0, kTabMul = 1, kTabSum = 2, kTabSub = 3, kTabProd = 4 };
+struct ElimTableOp {
+    uint8_t kind;
+    int dst, a, b;     // row: a = row index
+    int col;           // sum, sub: the column's place in the elimination order
+};
+
 struct ElimPlan {
     int n = 0, k = 0, h = 0;          // k low columns summed out, h outer columns walked
     int low[kNMax] = {};              // low columns in elimination order (original indices)
     int outer[kNMax] = {};            // outer column at Gray position p (original index)
     int last = 0;                     // the column that never flips
-    int exp2[kNMax] = {};             // FP64: row i is walked as x_i 2^-exp2[i] (exact scaling, |x_i| <= 1)
+    int exp2[kNMax] = {};             // FP64: row i is walked as x_i 2^-exp2[i] (elim_row_bits)
     int scale = 0;                    // FP64: sum of exp2: the walk's sum times 2^scale is the true one
     std::vector<ElimOp> ops;
     int result = 0;                   // the value that holds the step's signed sum
     std::vector<double> bound;        // exact: a bound of each value's magnitude (n + ops entries)
+    std::vector<ElimTable> tables;    // 0..n-1: x
+    std::vector<ElimTableOp> tops;
+    std::vector<int> factors;         // the step's sum is the product of these single values
+    double table_ops = 0.0;           // operations of the table program
     double ops_per_step = 0.0;        // counted operations per Gray step, flips and accumulation included
 };
 
@@ -56,6 +75,8 @@ struct ElimLimits {
     int max_ops = 1200;               // operations of a step's program
     double full_blocks = 19456.0;     // outer steps that fill the GPU: fewer take as long as these
     int candidates = kNMax;           // low columns tried per round of the search
+    bool allow_none = false;          // k = 0 (a full product per step) is a plan too
+    bool tables_only = false;         // write the program by tables only
 };
 
 // Picks the low columns among the first `free_cols` positions of col_order
@@ -65,10 +86,11 @@ struct ElimLimits {
 bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double range_log2, const ElimLimits &lim,
                ElimPlan &out);
 
-// The FP32 sum of |terms| walks every row's magnitude 2^bits above |x_i| <= 1,
-// so that a product of n of them, summed over 2^(k+3) terms, neither overflows
-// nor drifts into FP32's subnormals.
-inline int elim_abs_bits(int n, int k) { return std::max(0, std::min(8, (120 - k) / n)); }
+// FP64 rows are scaled by powers of two (exactly) to |x_i| <= 2^bits, so that a
+// product of n of them, summed over 2^(k+3) terms, neither leaves FP32's range
+// (the sum of |terms|) nor drifts into its subnormals, whatever the rows' own
+// magnitudes.
+inline int elim_row_bits(int n, int k) { return std::max(0, std::min(8, (120 - k) / n)); }
 
 // The CUDA C++ of the generated kernel (limbs 0: FP64, else the exact ring).
 std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want_abs);

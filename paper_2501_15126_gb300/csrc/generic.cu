@@ -6,6 +6,7 @@
 
 #include "core.cuh"
 #include "kernels.hpp"
+#include "vm.hpp"
 
 namespace pk {
 
@@ -142,6 +143,7 @@ GenericFns generic_fns_r160(int nmax, int fold);
 GenericFns generic_fns_r192(int nmax, int fold);
 
 GenericFns generic_fns(int nmax, int kind) {
+    if (nmax < 16) return vm_fns(kind);   // shared-memory classes of the eliminated walk
     const int limbs = kind >> 1, fold = kind & 1;
     switch (limbs) {
     case 0: return fold ? generic_fns_dd(nmax) : generic_fns_f64(nmax);

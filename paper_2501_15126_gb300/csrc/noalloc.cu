@@ -86,15 +86,31 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     const int n = P.m.n;
     P.engine = PERM_ENGINE_GENERIC;
     P.words = result_words(P.arith);
-    const int nmax = nmax_bucket(n);
-    P.nmax = nmax;
-    P.gf = generic_fns(nmax, P.kind());
-    if (!P.gf.walk) return failed(fail(PERM_ERR_INTERNAL, "no generic kernel"));
-    const size_t img_bytes = devmat_bytes_for(P.L, P.img_kind(), nmax);
-    if (img_bytes > kImageBytes) return failed(fail(PERM_ERR_INTERNAL, "image too large for the scratch array"));
     const uint64_t max_tasks = (kNoAllocScratchBytes - kOffTasks) / (8ull * P.words);
+    if (n > 8 && chunk_log2_that_fits(P, max_tasks, kBlockLog2) < 0)
+        return failed(fail(PERM_ERR_SIZE, "range too long (or its ends too finely aligned) for the scratch array"));
     cudaError_t e;
     cudaFuncAttributes attr;
+    int bps = 0;
+    size_t img_bytes = 0;
+    // the eliminated walk where its image and task results fit the array
+    bool vm = n > 8 && vm_prepare(P, kVmFullBlocks, 9) && P.vm_img.size() <= kImageBytes;
+    if (vm) {
+        P.gf = generic_fns(P.family_nmax(), P.family_kind());
+        if (!P.gf.walk) return failed(fail(PERM_ERR_INTERNAL, "no generic kernel"));
+        if ((e = P.gf.occ(32, P.vm_bytes, &bps)) != cudaSuccess) return failed(cuda_fail(e, "occupancy"));
+        choose_launch_elim(P, bps > 0 ? bps : 1, 32);
+        vm = P.ntasks <= max_tasks;
+    }
+    if (!vm) {
+        P.vm = P.use_elim = false;
+        adopt_elim(P);
+        P.gf = generic_fns(nmax_bucket(n), P.kind());
+        if (!P.gf.walk) return failed(fail(PERM_ERR_INTERNAL, "no generic kernel"));
+        img_bytes = devmat_bytes_for(P.L, P.img_kind(), nmax_bucket(n));
+        if (img_bytes > kImageBytes) return failed(fail(PERM_ERR_INTERNAL, "image too large for the scratch array"));
+    }
+    P.nmax = P.family_nmax();
     if ((e = P.gf.attr(&attr)) != cudaSuccess) return failed(cuda_fail(e, "cudaFuncGetAttributes"));
     P.regs = attr.numRegs;
     unsigned char *d_tasks = scratch + kOffTasks;
@@ -107,8 +123,7 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
         P.block = 256;
         P.grid = (int)((P.g_hi - P.g_lo + 255) / 256);
         P.ntasks = (uint64_t)P.grid;
-    } else {
-        int bps = 0;
+    } else if (!vm) {
         if ((e = P.gf.occ(256, img_bytes, &bps)) != cudaSuccess) return failed(cuda_fail(e, "occupancy"));
         perm_status_t s = choose_launch(P, P.gf.block_log2, bps > 0 ? bps : 1, 256);
         if (s != PERM_OK) return failed(s);
@@ -124,7 +139,8 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     if (P.ntasks > max_tasks) return failed(fail(PERM_ERR_SIZE, "too many tasks for the scratch array"));
 
     alignas(16) unsigned char image[kImageBytes];
-    build_devmat_into(P.m, P.L, P.img_kind(), nmax, image);
+    if (vm) std::memcpy(image, P.vm_img.data(), img_bytes = P.vm_img.size());
+    else build_devmat_into(P.m, P.L, P.img_kind(), P.nmax, image);
     if ((e = cudaMemcpyAsync(scratch + kOffImage, image, img_bytes, cudaMemcpyHostToDevice, st_)) != cudaSuccess)
         return failed(cuda_fail(e, "cudaMemcpyAsync(image)"));
     if ((e = cudaMemsetAsync(scratch + kOffCounters, 0, kOffResult + 32, st_)) != cudaSuccess)
@@ -150,7 +166,7 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
         ba.task_counter = reinterpret_cast<unsigned long long *>(d_counters);
         ba.task_out = reinterpret_cast<unsigned long long *>(d_tasks);
         ba.skip_counter = reinterpret_cast<unsigned long long *>(d_counters + 1);
-        ba.slot_bytes = img_bytes;
+        ba.slot_bytes = vm ? P.vm_bytes : img_bytes;
         ba.nmat = 1;
         ba.zero_skip = P.opts.zero_skip ? 0 : 1;
         ba.timeout_ns = (unsigned long long)std::max(0, P.opts.timeout_ms) * 1000000ull;

@@ -9,6 +9,7 @@
 
 #include "codegen.hpp"
 #include "elim.hpp"
+#include "vm.hpp"
 #include "host.hpp"
 #include "kernels.hpp"
 
@@ -59,6 +60,13 @@ struct perm_plan_s {
     bool use_elim = false;    // the walk sums out low columns (elim.hpp); chunks count outer Gray indices
     perm::ElimPlan elim;
     int val_shift = 0;        // FP64: the walk's sum is the true one times 2^-val_shift
+    bool vm = false;          // generic engine: the eliminated walk from a program image (vm.h)
+    std::vector<unsigned char> vm_img;
+    size_t vm_bytes = 0;      // per-warp shared memory: the image and its value slots
+    // kernel family of the generic engine: an NMAX bucket of the chained walk, or
+    // the eliminated walk's shared-memory class
+    int family_nmax() const;
+    int family_kind() const { return vm ? (dd ? perm::kKindDD : 2 * limbs) : kind(); }
     int kind() const { return dd ? perm::kKindDD : 2 * limbs + (fold ? 1 : 0); }   // generic kernel family
     int img_kind() const { return dd ? perm::kImgDD : (arith ? perm::kImgInt : perm::kImgF64); }   // matrix image layout
     uint64_t total = 0;       // 2^(n-1)
@@ -125,6 +133,8 @@ perm_status_t finish_raw(const perm_plan_s &P, const uint64_t *raw, perm_result_
 // perm_result_t.zero_skip_frac from the walk's skip counter
 double zero_skip_fraction(const perm_plan_s &P, uint64_t skipped);
 int nmax_bucket(int n);
+// x0_r of the double-double path as an exact pair (hi, lo).
+void x0_dd(const Matrix &m, int r, int last, double *hi_out, double *lo_out);
 // Matrix images; img is kImgF64, kImgInt or kImgDD.
 void build_devmat(const Matrix &m, const Layout &L, int img, int nmax, std::vector<unsigned char> &img_out);
 size_t devmat_bytes(int img, int nmax, int nnz);
@@ -138,6 +148,17 @@ perm_status_t choose_launch(perm_plan_s &P, int block_log2, int blocks_per_sm, i
 // chunks and grid.
 bool elim_allowed(const perm_plan_s &P);
 int range_free_cols(const perm_plan_s &P);
+// Plans the eliminated walk of the precompiled kernels and builds its image
+// (P.vm, P.use_elim): full_blocks as in ElimLimits.  vm_rebuild writes the image
+// again for the plan's current arithmetic (a double-double rerun).
+constexpr double kVmFullBlocks = 16384.0;   // single matrices: outer steps that fill the GPU
+constexpr double kVmFullBlocksShared = 64.0;   // batch and serving: other matrices fill it
+// Below min_n the chained walk takes less time than the planning.
+constexpr int kVmMinBatch = 19, kVmMinServe = 22;
+bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n);
+bool vm_rebuild(perm_plan_s &P);
+// Task chunks of a matrix that shares a launch with others: outer steps per lane.
+void choose_shared_chunks(perm_plan_s &P, int max_tasks_log2);
 constexpr int kElimWidth = 5;   // generated kernels: tables of at most 2^5 entries
 void codegen_choose_elim(perm_plan_s &P, int max_width);
 void adopt_elim(perm_plan_s &P);

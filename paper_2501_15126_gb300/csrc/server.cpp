@@ -57,6 +57,7 @@ constexpr int kServeChunkLog2 = 12;           // chunk length target: tasks of 2
 constexpr int kAdmitScan = 256;               // queued requests looked at past a blocked one
 constexpr double kNoSkipAfterMs = 200.0;      // a request blocked this long stops being overtaken
 constexpr size_t kQueueMax = 1 << 20;
+constexpr size_t kVmImageCap = 24 * 1024;     // one image slot of an eliminated-walk family
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -81,7 +82,7 @@ struct Request {
     int slot = -1;
     uint64_t ntasks = 0, next_task = 0, done_tasks = 0;
     uint64_t out_offset = 0;    // first task of the request's result range in the family pool
-    size_t img_bytes = 0;       // size of the request's matrix image
+    size_t slot_bytes = 0;      // per-warp shared memory of the request (its image, and value slots)
     double t_submit = 0.0;
     int inflight_waves = 0;
     bool failed = false;
@@ -120,6 +121,9 @@ struct Family {
     int nmax = 0, kind = 0, arith = 0, words = 3, K_target = 14;   // kind: generic kernel family
     int img = 0;                                                  // image layout (kImgF64, kImgInt, kImgDD)
     GenericFns gf;
+    bool vm = false;                       // the eliminated walk (vm.hpp)
+    int block = 256;
+    size_t image_cap = 0;                  // bytes of one image slot
     int grid_max = 1;
     unsigned char *d_images = nullptr;
     uint64_t *d_pool = nullptr;
@@ -185,7 +189,8 @@ struct perm_server_s {
     double t_first = 0.0, t_last = 0.0;
     perm_status_t init_status = PERM_OK;
 
-    static int family_index(int nmax, int kind) { return (nmax / 16 - 1) * 14 + kind; }
+    // chained walk: 16, 32, 48 -> 0..41; the eliminated walk's classes 1..3 after them
+    static int family_index(int nmax, int kind) { return (nmax < 16 ? nmax + 2 : nmax / 16 - 1) * 14 + kind; }
 
     perm_status_t init_device() {   // on the creating thread, with `device` current
         cudaError_t e;
@@ -208,7 +213,7 @@ struct perm_server_s {
             if ((e = cudaMallocHost(&f.h_res, 32 * (size_t)maxn)) != cudaSuccess) return cuda_fail(e, "pinned");
             if ((e = cudaMalloc(&f.d_res, 32 * (size_t)maxn)) != cudaSuccess) return cuda_fail(e, "res");
         }
-        fam.resize(42);
+        fam.resize(84);
         return PERM_OK;
     }
 
@@ -223,13 +228,16 @@ struct perm_server_s {
         F.img = kind == kKindDD ? kImgDD : (F.arith ? kImgInt : kImgF64);
         F.gf = generic_fns(nmax, kind);
         if (!F.gf.walk) return fail(PERM_ERR_INTERNAL, "no generic kernel for this family");
-        F.K_target = tuned_chunk_log2(nmax, kind);
+        F.vm = nmax < 16;
+        F.block = F.vm ? 32 : 256;
+        F.image_cap = F.vm ? kVmImageCap : F.gf.devmat_bytes;
+        if (!F.vm) F.K_target = tuned_chunk_log2(nmax, kind);
         int bps = 0;
-        cudaError_t e = F.gf.occ(256, F.gf.devmat_bytes, &bps);
+        cudaError_t e = F.gf.occ(F.block, F.image_cap, &bps);
         if (e != cudaSuccess) return cuda_fail(e, "occupancy");
         F.grid_max = kSMCount * std::max(bps, 1);
         const int slots = opts.max_inflight;
-        if ((e = cudaMalloc(&F.d_images, (size_t)slots * F.gf.devmat_bytes)) != cudaSuccess) return cuda_fail(e, "images");
+        if ((e = cudaMalloc(&F.d_images, (size_t)slots * F.image_cap)) != cudaSuccess) return cuda_fail(e, "images");
         // result pool: every slot's largest request at once would be too much; size it for the step budget
         F.pool_tasks = std::max<uint64_t>(1ull << 21, (uint64_t)(step_budget / std::ldexp(1.0, F.K_target + 5)) * 2 + 4096);
         F.pool_tasks = std::min<uint64_t>(F.pool_tasks, 1ull << 23);
@@ -290,17 +298,19 @@ struct perm_server_s {
             Family &F = fam[r->family];
             if (F.free_slots.empty()) return false;
             // at most 2^20 tasks per request, so the largest n fits the result pool
-            const int K = batch_chunk_log2(P.m.n, F.gf.block_log2, std::max(kServeChunkLog2, P.m.n - 26));
-            const uint64_t chunks = P.total >> K;
-            const uint64_t ntasks = (chunks + 31) / 32;
+            if (F.vm) {
+                choose_shared_chunks(P, 20);
+            } else {
+                P.K = batch_chunk_log2(P.m.n, F.gf.block_log2, std::max(kServeChunkLog2, P.m.n - 26));
+                P.chunk_lo = 0;
+                P.chunk_hi = P.total >> P.K;
+                P.ntasks = (P.chunk_hi + 31) / 32;
+            }
+            const uint64_t ntasks = P.ntasks;
             uint64_t off = 0;
             if (!F.ranges.alloc(ntasks, &off)) return false;
             r->slot = F.free_slots.back();
             F.free_slots.pop_back();
-            P.K = K;
-            P.chunk_lo = 0;
-            P.chunk_hi = chunks;
-            P.ntasks = ntasks;
             P.engine = PERM_ENGINE_GENERIC;
             P.gf = F.gf;
             P.nmax = F.nmax;
@@ -308,10 +318,11 @@ struct perm_server_s {
             r->out_offset = off;
             // the image goes up on the aux stream; every wave waits for the uploads made so far
             std::vector<unsigned char> img;
-            build_devmat(P.m, P.L, F.img, F.nmax, img);
-            r->img_bytes = img.size();
+            if (F.vm) img.swap(P.vm_img);
+            else build_devmat(P.m, P.L, F.img, F.nmax, img);
+            r->slot_bytes = F.vm ? P.vm_bytes : img.size();
             const cudaError_t e = debug_fail(kSiteUpload) ? cudaErrorInvalidValue
-                                  : cudaMemcpyAsync(F.d_images + (size_t)r->slot * F.gf.devmat_bytes, img.data(),
+                                  : cudaMemcpyAsync(F.d_images + (size_t)r->slot * F.image_cap, img.data(),
                                                     img.size(), cudaMemcpyHostToDevice, aux);
             if (e != cudaSuccess) fail_request(r, cuda_fail(e, "serving: image upload"));
         }
@@ -372,7 +383,7 @@ struct perm_server_s {
                 if (r->family != fi || r->failed) continue;
                 const uint64_t left = r->ntasks - r->next_task;
                 if (!left) continue;
-                const double task_steps = std::ldexp(32.0, r->P->K);
+                const double task_steps = r->P->vm ? std::ldexp(4.0 * r->P->elim.table_ops, r->P->K) : std::ldexp(32.0, r->P->K);
                 uint64_t take = pass == 0 ? std::min(left, kSmallShare) : left;
                 take = std::min<uint64_t>(take, std::max<uint64_t>(1, (uint64_t)(budget / task_steps)));
                 auto it = where.find(r);
@@ -400,7 +411,7 @@ struct perm_server_s {
             bm.chunk_lo = first * 32;
             bm.chunk_hi = std::min<uint64_t>((first + take) * 32, r->P->chunk_hi);
             bm.out_offset = r->out_offset + first;
-            bm.image = (int)((size_t)r->slot * F.gf.devmat_bytes / 16);
+            bm.image = (int)((size_t)r->slot * F.image_cap / 16);
             bm.K = r->P->K;
             bm.abs_shift = r->P->abs_shift;
             r->inflight_waves += 1;
@@ -422,7 +433,7 @@ struct perm_server_s {
         ba.task_out = reinterpret_cast<unsigned long long *>(F.d_pool);
         ba.skip_counter = nullptr;
         size_t slot_bytes = 16;
-        for (const Part &pt : w->parts) slot_bytes = std::max(slot_bytes, pt.req->img_bytes);
+        for (const Part &pt : w->parts) slot_bytes = std::max(slot_bytes, pt.req->slot_bytes);
         ba.slot_bytes = slot_bytes;
         ba.nmat = (int)w->parts.size();
         ba.zero_skip = 1;
@@ -430,10 +441,10 @@ struct perm_server_s {
         ba.deadline_word = nullptr;
         ba.abort_flag = nullptr;
         int bps = 1;
-        if (e == cudaSuccess) e = F.gf.occ(256, slot_bytes, &bps);
+        if (e == cudaSuccess) e = F.gf.occ(F.block, slot_bytes, &bps);
         const uint64_t grid_occ = (uint64_t)kSMCount * std::max(bps, 1);
-        const int grid = (int)std::min<uint64_t>(grid_occ, (t * 32 + 255) / 256);
-        if (e == cudaSuccess) e = debug_fail(kSiteWaveLaunch) ? cudaErrorLaunchFailure : F.gf.walk(ba, std::max(grid, 1), 256, st);
+        const int grid = (int)std::min<uint64_t>(grid_occ, (t * 32 + F.block - 1) / F.block);
+        if (e == cudaSuccess) e = debug_fail(kSiteWaveLaunch) ? cudaErrorLaunchFailure : F.gf.walk(ba, std::max(grid, 1), F.block, st);
         if (e == cudaSuccess) e = cudaEventRecord(w->done, st);
         if (e != cudaSuccess) {
             // nothing of this wave counts: its requests fail instead of
@@ -517,13 +528,17 @@ struct perm_server_s {
         steps_active -= (double)P.total;
         auto it = std::find(active.begin(), active.end(), r);
         if (it != active.end()) active.erase(it);
-        const int nmax = nmax_bucket(P.m.n);
         P.dd = true;
-        r->family = family_index(nmax, P.kind());
+        if (P.vm && (!vm_rebuild(P) || P.vm_img.size() > kVmImageCap)) {   // too many pair slots: the chained walk
+            P.vm = P.use_elim = false;
+            adopt_elim(P);
+        }
+        const int nmax = P.family_nmax(), kind = P.family_kind();
+        r->family = family_index(nmax, kind);
         r->slot = -1;
         r->ntasks = r->next_task = r->done_tasks = 0;
         r->inflight_waves = 0;
-        if (ensure_family(r->family, nmax, P.kind()) != PERM_OK) {
+        if (ensure_family(r->family, nmax, kind) != PERM_OK) {
             r->retired = true;   // holds nothing any more
             return false;
         }
@@ -639,7 +654,7 @@ struct perm_server_s {
                     Request *r = f.reqs[i];
                     perm_result_t res;
                     r->P->grid = fam[f.family].grid_max;
-                    r->P->block = 256;
+                    r->P->block = fam[f.family].block;
                     describe(*r->P, &res);
                     if (fs != PERM_OK) res.status = fs;
                     else finish_raw(*r->P, f.h_res + 4 * i, &res);
@@ -721,6 +736,12 @@ perm_status_t perm_submit(perm_server_t s, const perm_matrix_t *A, uint64_t *tic
     perm_status_t st = plan_prepare(A, &po, *r->P);
     if (st != PERM_OK) return st;
     perm_plan_s &P = *r->P;
+    // a server with a deadline keeps the chained walk, as a call with one does
+    if (!P.zero && s->opts.timeout_ms == 0 && vm_prepare(P, kVmFullBlocksShared, kVmMinServe) &&
+        P.vm_img.size() > kVmImageCap) {
+        P.vm = P.use_elim = false;
+        adopt_elim(P);
+    }
     r->t_submit = now_ms();
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->stop) return fail(PERM_ERR_CANCELLED, "server is shutting down");
@@ -738,9 +759,8 @@ perm_status_t perm_submit(perm_server_t s, const perm_matrix_t *A, uint64_t *tic
         return PERM_OK;
     }
     if (P.m.n > 8 && P.m.n <= 48) {
-        const int nmax = nmax_bucket(P.m.n);
-        raw->family = perm_server_s::family_index(nmax, P.kind());
-        st = s->ensure_family(raw->family, nmax, P.kind());
+        raw->family = perm_server_s::family_index(P.family_nmax(), P.family_kind());
+        st = s->ensure_family(raw->family, P.family_nmax(), P.family_kind());
         if (st != PERM_OK) { s->all.erase(raw->ticket); return st; }
     }
     s->queue.push_back(raw);

@@ -65,10 +65,9 @@ def compare(src, words, ao, lo, hi):
     s, sa = oracle.nw_range(ao, lo, hi)
     hi_w, lo_w, ab = np.array(words, dtype=np.uint64).view(np.float64)
     scale = int(re.search(r"int scale = (-?\d+);", src).group(1))
-    shift = int(re.search(r"int abs_shift = (-?\d+);", src).group(1))
     assert abs(np.ldexp(hi_w + lo_w, scale) - float(s)) <= 64 * n * U * float(sa)
     if "kAbs = true" in src:
-        assert abs(np.ldexp(ab, shift) - float(sa)) <= 1e-4 * float(sa)
+        assert abs(np.ldexp(ab, scale) - float(sa)) <= 1e-4 * float(sa)
 
 
 def scaled_rows(n, p, seed):
