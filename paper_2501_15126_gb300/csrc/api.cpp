@@ -453,14 +453,15 @@ static void codegen_layout(perm_plan_s &P) {
 // half the chain's counted operations per Gray step: a step's program has no
 // block start, vote or skip, so equal counts would already be even, and dense
 // patterns (J_30: nothing to share) stay with the chain.  Measured, chained ->
-// eliminated: n=36 p=0.15 FP64 368 -> 2.76 ms per permanent (6.5 -> 0.024
-// operations per Gray step), n=34 p=0.2 0/1 7.0 -> 0.79 ms, 2^30-step slices of
+// eliminated (tables of 2^5 entries): n=36 p=0.15 FP64 368 -> 2.76 ms per
+// permanent (6.5 -> 0.024 operations per Gray step), n=34 p=0.2 0/1 7.0 -> 0.79 ms, 2^30-step slices of
 // the n=48 band: exact 6.41 -> 0.127 ms, FP64 16.9 -> 0.153 ms.
 void codegen_choose_elim(perm_plan_s &P, int max_width) {
     P.use_elim = false;
     if (max_width < 2 || !elim_allowed(P) || P.zero_spans) return;
     ElimLimits lim;
     lim.max_width = max_width;
+    if (!P.m.is_int) lim.max_ops = 1600;   // about 0.65 s of NVRTC
     const double range = std::log2((double)(P.g_hi - P.g_lo));
     if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return;
     if (P.elim.ops_per_step > 0.5 * P.ops_per_step) return;
@@ -490,8 +491,8 @@ bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
     // call; n=28 p=0.4 0/1, whose rows share too much, stays with the chain (2.2 ms).
     // The chained walk's time in lane-operations of the whole GPU.  Alone, a walk
     // of fewer than 152 blocks' tasks (eight 32-chunk tasks of 2^8 steps, exact
-    // 2^6) leaves SMs idle; an exact chained step is about 90 instructions, an
-    // interpreted operation about 20.
+    // 2^6) leaves SMs idle; an exact chained step takes as long as nine operations
+    // of the precompiled program (n=28 p=0.3/0.4: 6.1e10 steps/s, 5.5e11 operations/s).
     const bool alone = full_blocks == kVmFullBlocks;
     const double ops = P.m.is_int ? 90.0 : n > 32 ? cost_per_step(P.L, false) : cost_per_step_dual(P.L, true);
     const double sms = alone ? std::min(152.0, std::max(1.0, std::exp2(range - (P.m.is_int ? 14.0 : 16.0)))) : 152.0;
@@ -504,7 +505,7 @@ bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
         lim.max_width = width;
         if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;
         const double steps = std::max(std::exp2(range - P.elim.k), full_blocks);
-        if ((P.elim.table_ops + 10.0) * (P.m.is_int ? 20.0 : 1.0) * steps > 0.9 * chain) return false;
+        if ((P.elim.table_ops + 10.0) * (P.m.is_int ? 10.0 : 1.0) * steps > 0.9 * chain) return false;
         P.vm = P.use_elim = true;
         if (vm_rebuild(P)) {
             adopt_elim(P);
@@ -1107,7 +1108,7 @@ perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, 
     perm_status_t st = plan_prepare(A, opts, P);
     if (st != PERM_OK) return st;
     codegen_layout(P);
-    codegen_choose_elim(P, kElimWidth);
+    codegen_choose_elim(P, elim_width(P));
     std::string src = P.use_elim ? elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs) : std::string();
     adopt_elim(P);
     if (k) *k = P.use_elim ? P.elim.k : 0;

@@ -552,6 +552,7 @@ struct CacheEntry {
 // size) is also built for 255 registers, both walk the same probe chunks on the
 // GPU, and the 128-register build is kept only if the two agree bit for bit.
 constexpr int kMaxLocalFrame = 512;
+constexpr int kMaxElimFrame = 4096;   // bytes per thread of an eliminated FP64 step
 
 std::mutex g_cache_mu;
 std::unordered_map<std::string, CacheEntry> g_cache;
@@ -712,19 +713,20 @@ perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
         P.ms_compile = 0.0;
         return true;
     };
-    // The eliminated walk, planned narrower while its kernel spills (255
-    // registers): FP64 steps tolerate a small frame (the FP64 pipe bounds
-    // them), exact ones none; then the chained walk.
+    // The eliminated walk, planned narrower while its kernel spills more than it
+    // may (255 registers): FP64 steps have some sixty issue slots per operation
+    // of the FP64 pipe, so spills to L1 cost them little; exact ones get none.
+    // Then the chained walk.
     perm_status_t st = PERM_OK;
     bool built = false;
-    for (int width = kElimWidth; width >= 2 && !built; --width) {
+    for (int width = elim_width(P); width >= 2 && !built; --width) {
         codegen_choose_elim(P, width);
         if (!P.use_elim) break;
         const std::string src = elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs);
         if (cached(src)) { adopt_elim(P); return PERM_OK; }
         st = compile_and_load(src, ce, err, 0);
         if (st != PERM_OK) return st;
-        if (ce.local_bytes <= (P.arith == 0 ? kMaxLocalFrame : 0)) {
+        if (ce.local_bytes <= (P.arith == 0 ? kMaxElimFrame : 0)) {
             built = true;
         } else {
             driver().moduleUnload(ce.module);

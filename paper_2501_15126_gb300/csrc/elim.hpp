@@ -73,7 +73,7 @@ struct ElimPlan {
 struct ElimLimits {
     int max_width = 5;                // tables of at most 2^max_width entries while a column is summed out
     int max_ops = 1200;               // operations of a step's program
-    double full_blocks = 19456.0;     // outer steps that fill the GPU: fewer take as long as these
+    double full_blocks = 32768.0;     // outer steps that fill the GPU: fewer take as long as these
     int candidates = kNMax;           // low columns tried per round of the search
     bool allow_none = false;          // k = 0 (a full product per step) is a plan too
     bool tables_only = false;         // write the program by tables only

@@ -154,12 +154,18 @@ int range_free_cols(const perm_plan_s &P);
 constexpr double kVmFullBlocks = 16384.0;   // single matrices: outer steps that fill the GPU
 constexpr double kVmFullBlocksShared = 64.0;   // batch and serving: other matrices fill it
 // Below min_n the chained walk takes less time than the planning.
-constexpr int kVmMinBatch = 19, kVmMinServe = 22;
+constexpr int kVmMinBatch = 9, kVmMinServe = 22;
 bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n);
 bool vm_rebuild(perm_plan_s &P);
 // Task chunks of a matrix that shares a launch with others: outer steps per lane.
 void choose_shared_chunks(perm_plan_s &P, int max_tasks_log2);
-constexpr int kElimWidth = 5;   // generated kernels: tables of at most 2^5 entries
+// Generated kernels: the widest tables tried first.  FP64 steps are bound by the
+// FP64 pipe, so fewer operations pay even when the tables spill (the n=36
+// workload: 2^5 entries 1.72 ms, 2^6 1.42, 2^7 0.91, 2^8 0.89 ms but 1-2.5 s of
+// compilation at n = 32-40); with sums of |terms| compilation takes twice as
+// long, and stops at 2^6.  Exact steps are bound by their instructions, which
+// spills add to (n=34 p=0.2 0/1: 0.98 ms at 2^5, 1.63 at 2^6).
+inline int elim_width(const perm_plan_s &P) { return P.m.is_int ? 5 : P.want_abs ? 6 : 7; }
 void codegen_choose_elim(perm_plan_s &P, int max_width);
 void adopt_elim(perm_plan_s &P);
 void choose_launch_elim(perm_plan_s &P, int blocks_per_sm, int block);
