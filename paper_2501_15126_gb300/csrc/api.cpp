@@ -643,6 +643,7 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
             return cuda_fail(e, "cudaMemcpy(batch table)");
     }
     if ((e = cudaMallocHost(&P.h_res, 8 * 8)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
+    if (P.fused() && (e = cudaMemset(P.d_ws, 0, 8 * 8)) != cudaSuccess) return cuda_fail(e, "cudaMemset(counters)");
     if ((e = cudaEventCreate(&P.ev0)) != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
     if ((e = cudaEventCreate(&P.ev1)) != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
     P.ms_plan += now_ms() - t0 - P.ms_compile;
@@ -654,14 +655,21 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
 // replayed graph is timed by events around its launch instead.
 perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(P.d_ws, 0, 8 * 8, st)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    const bool fused = P.fused();   // one launch: counters are clear, the walk writes h_res
+    if (!fused && (e = cudaMemsetAsync(P.d_ws, 0, 8 * 8, st)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     uint64_t *task_out = P.d_ws + kWsTaskOut;
+    pk::FinishArgs finish;
+    finish.host = fused ? reinterpret_cast<unsigned long long *>(P.h_res) : nullptr;
+    finish.ws = reinterpret_cast<unsigned long long *>(P.d_ws);
+    finish.task_out = reinterpret_cast<unsigned long long *>(task_out);
+    finish.ntasks = P.ntasks;
     if (record_events && (e = cudaEventRecord(P.ev0, st)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
     if (P.direct) {
         e = P.gf.direct(P.d_devmat, P.g_lo, P.g_hi, task_out, P.grid, P.block, st, P.abs_shift);
         if (e != cudaSuccess) return cuda_fail(e, "direct kernel launch");
     } else if (P.engine == PERM_ENGINE_XSHARED) {
         pk::WalkArgs wa;
+        wa.finish = finish;
         wa.chunk_lo = P.chunk_lo;
         wa.chunk_hi = P.chunk_hi;
         wa.ntasks = P.ntasks;
@@ -679,6 +687,7 @@ perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
         if (e != cudaSuccess) return cuda_fail(e, "walk kernel launch");
     } else if (P.engine == PERM_ENGINE_GENERIC) {
         pk::BatchArgs ba;
+        ba.finish = finish;
         ba.mats = reinterpret_cast<const pk::BatchMat *>(P.d_ws + kWsBatchMat);
         ba.devmats = P.d_devmat;
         ba.ntasks = P.ntasks;
@@ -695,6 +704,7 @@ perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
         if (e != cudaSuccess) return cuda_fail(e, "walk kernel launch");
     } else {
         pk::WalkArgs wa;
+        wa.finish = finish;
         wa.chunk_lo = P.chunk_lo;
         wa.chunk_hi = P.chunk_hi;
         wa.ntasks = P.ntasks;
@@ -708,6 +718,10 @@ perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
         wa.abort_flag = reinterpret_cast<unsigned int *>(P.d_ws + kWsAbort);
         e = debug_fail(kSiteLaunch) ? cudaErrorLaunchFailure : codegen_launch(P, wa, st);
         if (e != cudaSuccess) return cuda_fail(e, "walk kernel launch");
+    }
+    if (fused) {
+        if (record_events && (e = cudaEventRecord(P.ev1, st)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
+        return PERM_OK;
     }
     if ((e = reduce_launch(P.arith, task_out, P.ntasks, P.d_ws + 2, P.d_ws + kWsReduced, st)) != cudaSuccess)
         return cuda_fail(e, "reduce kernel launch");
@@ -979,7 +993,8 @@ perm_status_t perm_compute(perm_plan_t plan, void *stream, perm_result_t *out) {
 static perm_status_t compute_one(perm_plan_t plan, void *stream, perm_result_t *out) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (!plan->zero) {
-        const bool use_graph = !(plan->opts.flags & PERM_FLAG_NO_GRAPH) && plan->computes >= 1;
+        // (a fused walk is one launch already)
+        const bool use_graph = !(plan->opts.flags & PERM_FLAG_NO_GRAPH) && plan->computes >= 1 && !plan->fused();
         if (use_graph && !plan->graph && !plan->graph_failed) plan->graph_failed = !capture_graph(*plan);
         perm_status_t s = PERM_OK;
         if (use_graph && plan->graph) {

@@ -127,6 +127,7 @@ int BatchGroup::launch(cudaStream_t st, int zero_skip) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(d_counters, 0, 32, st)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     pk::BatchArgs ba;
+    ba.finish = pk::FinishArgs();
     ba.mats = d_mats;
     ba.devmats = d_images;
     ba.ntasks = ntasks;

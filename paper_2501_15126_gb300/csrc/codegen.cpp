@@ -33,9 +33,10 @@
 #include "codegen.hpp"
 #include "plan.hpp"
 
-// Embedded copies of core.cuh and devmat.h (generated at build time).
+// Embedded copies of core.cuh, devmat.h and finish.cuh (generated at build time).
 extern const char *perm_embedded_core_cuh;
 extern const char *perm_embedded_devmat_h;
+extern const char *perm_embedded_finish_cuh;
 
 namespace perm {
 
@@ -579,9 +580,9 @@ perm_status_t compile_and_load(const std::string &src, CacheEntry &ce, std::stri
     Driver &d = driver();
     if (debug_fail(kSiteNvrtc)) { err = "NVRTC compile failed (injected by perm_debug_inject_failures)"; return PERM_ERR_NVRTC; }
     nvrtcProgram prog;
-    const char *hdr_src[2] = {perm_embedded_core_cuh, perm_embedded_devmat_h};
-    const char *hdr_name[2] = {"core.cuh", "devmat.h"};
-    nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), "perm_walk.cu", 2, hdr_src, hdr_name);
+    const char *hdr_src[3] = {perm_embedded_core_cuh, perm_embedded_devmat_h, perm_embedded_finish_cuh};
+    const char *hdr_name[3] = {"core.cuh", "devmat.h", "finish.cuh"};
+    nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), "perm_walk.cu", 3, hdr_src, hdr_name);
     if (r != NVRTC_SUCCESS) { err = std::string("nvrtcCreateProgram: ") + nvrtcGetErrorString(r); return PERM_ERR_NVRTC; }
     const char *opts[] = {"--gpu-architecture=sm_103a", "-std=c++17", "-lineinfo", "--device-as-default-execution-space"};
     r = nvrtcCompileProgram(prog, 4, opts);
@@ -652,6 +653,7 @@ perm_status_t same_on_probe(const perm_plan_s &P, const CacheEntry &a, const Cac
         e = cudaMemsetAsync(ws, 0, 16 * 8, st);
         if (e != cudaSuccess) break;
         pk::WalkArgs wa;
+        wa.finish = pk::FinishArgs();
         wa.chunk_lo = 0;
         wa.chunk_hi = chunks;
         wa.ntasks = ntasks;

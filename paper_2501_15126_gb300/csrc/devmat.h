@@ -6,6 +6,14 @@
 
 namespace pk {
 
+// The end of a plan's walk in the walk's own launch (finish.cuh).
+struct FinishArgs {
+    unsigned long long *host;           // result words in pinned host memory; null: a reduction kernel follows
+    unsigned long long *ws;             // the plan's workspace words
+    unsigned long long *task_out;
+    unsigned long long ntasks;
+};
+
 // Launch arguments of one Gray-code walk (see core.cuh).
 struct WalkArgs {
     unsigned long long chunk_lo;        // first chunk index (in units of 2^K Gray indices)
@@ -19,6 +27,7 @@ struct WalkArgs {
     unsigned long long timeout_ns;      // device-side deadline, counted from the first task fetch (0 = none)
     unsigned long long *deadline_word;  // zeroed before the launch; the first warp stores its deadline
     unsigned int *abort_flag;           // set to 1 by a warp that stopped at the deadline
+    FinishArgs finish;                  // eliminated walks only
 };
 
 // One entry of a generic (multi-matrix) walk: the launch's tasks
@@ -53,6 +62,7 @@ struct BatchArgs {
     unsigned long long timeout_ns;      // device-side deadline, counted from the first task fetch (0 = none)
     unsigned long long *deadline_word;  // zeroed before the launch; the first warp stores its deadline
     unsigned int *abort_flag;           // set to 1 by a warp that stopped at the deadline
+    FinishArgs finish;                  // eliminated walks only
 };
 
 // The ordered matrix as the generic kernels read it (a variable-length

@@ -439,7 +439,7 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
     std::ostringstream o;
     o << "// generated: eliminated permanent walk for one " << n << "x" << n << " matrix\n";
     o << "// low columns k=" << E.k << " outer columns h=" << E.h << " operations per outer step " << E.ops.size() << "\n";
-    o << "#include \"core.cuh\"\n\nnamespace pk {\n";
+    o << "#include \"core.cuh\"\n#ifndef PERM_HOST_EMULATION\n#include \"finish.cuh\"\n#endif\n\nnamespace pk {\n";
     if (fp) o << "typedef ArithF64 A;\n";
     else o << "typedef ArithExact<" << limbs << "> A;\n";
     o << "struct ElimPol {\n    static constexpr int NX = " << n << ";\n";
@@ -549,7 +549,8 @@ std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want
     // One block per SM (255 registers): FP64 steps are bound by the FP64 pipe (2
     // lane-operations per clock and SM), which eight warps keep 85 % busy (ncu).
     o << "extern \"C\" __global__ void __launch_bounds__(256, 1) perm_walk(pk::WalkArgs wa, void *) {\n";
-    o << "    pk::elim_tasks<pk::ElimPol, pk::A>(wa);\n}\n";
+    o << "    pk::elim_tasks<pk::ElimPol, pk::A>(wa);\n";
+    o << "#ifndef PERM_HOST_EMULATION\n    pk::finish_walk<pk::A>(wa.finish);\n#endif\n}\n";
     return o.str();
 }
 

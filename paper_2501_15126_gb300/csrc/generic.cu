@@ -4,7 +4,7 @@
 
 #include <cuda_runtime.h>
 
-#include "core.cuh"
+#include "finish.cuh"
 #include "kernels.hpp"
 #include "vm.hpp"
 
@@ -18,21 +18,8 @@ namespace pk {
 // 25-38 us in its shuffle trees; blocks of 128 threads over the whole GPU
 // spend a few.)
 template <class A>
-__device__ __forceinline__ typename A::Acc block_sum(typename A::Acc acc, u64 *sh) {
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) acc = A::acc_add(acc, A::shfl_down(acc, d));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    if (lane == 0) A::acc_store(sh + warp * A::ACC_WORDS, acc);
-    __syncthreads();
-    acc = A::acc_load(sh);
-    for (int w = 1; w < nw; ++w) acc = A::acc_add(acc, A::acc_load(sh + w * A::ACC_WORDS));
-    return acc;   // (in every thread)
-}
-
-template <class A>
 __device__ __forceinline__ void reduce_tasks(u64 *task_out, u64 ntasks, u64 per, u64 *result, u64 *done_blocks) {
     __shared__ u64 sh[32 * 6];
-    __shared__ int last;
     typename A::Acc acc = A::acc_zero();
     const u64 b = blockIdx.x * per, e = b + per < ntasks ? b + per : ntasks;
     for (u64 t = b + threadIdx.x; t < e; t += blockDim.x)
@@ -42,21 +29,11 @@ __device__ __forceinline__ void reduce_tasks(u64 *task_out, u64 ntasks, u64 per,
         if (threadIdx.x == 0) A::acc_store(result, A::acc_norm(acc));
         return;
     }
-    if (threadIdx.x == 0) {
-        A::acc_store(task_out + b * (u64)A::ACC_WORDS, acc);
-        __threadfence();
-        last = atomicAdd(done_blocks, 1ull) == gridDim.x - 1;
-        __threadfence();
-    }
-    __syncthreads();
-    if (!last) return;
+    if (threadIdx.x == 0) A::acc_store(task_out + b * (u64)A::ACC_WORDS, acc);
+    if (!last_block(done_blocks)) return;
     acc = A::acc_zero();
-    for (u64 k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
-        u64 w[A::ACC_WORDS];
-#pragma unroll
-        for (int i = 0; i < A::ACC_WORDS; ++i) w[i] = ((volatile u64 *)task_out)[k * per * (u64)A::ACC_WORDS + i];
-        acc = A::acc_add(acc, A::acc_load(w));
-    }
+    for (u64 k = threadIdx.x; k < gridDim.x; k += blockDim.x)
+        acc = A::acc_add(acc, acc_load_l2<A>(task_out + k * per * (u64)A::ACC_WORDS));
     acc = block_sum<A>(acc, sh);
     if (threadIdx.x == 0) A::acc_store(result, A::acc_norm(acc));
 }

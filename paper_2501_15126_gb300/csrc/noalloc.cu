@@ -38,6 +38,8 @@ constexpr size_t kImageBytes = 20480;
 constexpr size_t kOffTasks = kOffImage + kImageBytes;   // per-task partial sums
 constexpr int kMaxDevices = 64;
 static_assert(sizeof(pk::BatchMat) <= kOffImage - kOffBatchMat, "task table entry");
+// (finish.cuh writes words 1..6 from two words before the result)
+static_assert(kOffResult - 16 + 7 * 8 <= kOffBatchMat && kOffResult >= 16 + 8 * 8, "result words");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
@@ -138,28 +140,38 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     }
     if (P.ntasks > max_tasks) return failed(fail(PERM_ERR_SIZE, "too many tasks for the scratch array"));
 
-    alignas(16) unsigned char image[kImageBytes];
-    if (vm) std::memcpy(image, P.vm_img.data(), img_bytes = P.vm_img.size());
-    else build_devmat_into(P.m, P.L, P.img_kind(), P.nmax, image);
-    if ((e = cudaMemcpyAsync(scratch + kOffImage, image, img_bytes, cudaMemcpyHostToDevice, st_)) != cudaSuccess)
-        return failed(cuda_fail(e, "cudaMemcpyAsync(image)"));
-    if ((e = cudaMemsetAsync(scratch + kOffCounters, 0, kOffResult + 32, st_)) != cudaSuccess)
-        return failed(cuda_fail(e, "cudaMemsetAsync(counters)"));
-    if (P.direct) {
-        e = P.gf.direct(scratch + kOffImage, P.g_lo, P.g_hi, reinterpret_cast<uint64_t *>(d_tasks), P.grid, P.block,
-                        st_, P.abs_shift);
-        if (e != cudaSuccess) return failed(cuda_fail(e, "direct kernel launch"));
-    } else {
+    // counters and result cleared, task table and image: one upload (its source is
+    // on the stack: the copy is staged before cudaMemcpyAsync returns)
+    alignas(16) unsigned char up[kOffImage + kImageBytes];
+    std::memset(up, 0, kOffImage);
+    if (vm) std::memcpy(up + kOffImage, P.vm_img.data(), img_bytes = P.vm_img.size());
+    else build_devmat_into(P.m, P.L, P.img_kind(), P.nmax, up + kOffImage);
+    if (!P.direct) {
         pk::BatchMat bm;
         std::memset(&bm, 0, sizeof(bm));
         bm.chunk_lo = P.chunk_lo;
         bm.chunk_hi = P.chunk_hi;
         bm.K = P.K;
         bm.abs_shift = P.abs_shift;
-        // a stack source: the copy is staged before cudaMemcpyAsync returns
-        if ((e = cudaMemcpyAsync(scratch + kOffBatchMat, &bm, sizeof(bm), cudaMemcpyHostToDevice, st_)) != cudaSuccess)
-            return failed(cuda_fail(e, "cudaMemcpyAsync(task table)"));
+        std::memcpy(up + kOffBatchMat, &bm, sizeof(bm));
+    }
+    if ((e = cudaMemcpyAsync(scratch, up, kOffImage + img_bytes, cudaMemcpyHostToDevice, st_)) != cudaSuccess)
+        return failed(cuda_fail(e, "cudaMemcpyAsync(counters, task table, image)"));
+    bool fused = false;
+    if (P.direct) {
+        e = P.gf.direct(scratch + kOffImage, P.g_lo, P.g_hi, reinterpret_cast<uint64_t *>(d_tasks), P.grid, P.block,
+                        st_, P.abs_shift);
+        if (e != cudaSuccess) return failed(cuda_fail(e, "direct kernel launch"));
+    } else {
         pk::BatchArgs ba;
+        ba.finish = pk::FinishArgs();
+        fused = vm && P.ntasks <= kFusedTasks;
+        if (fused) {   // the walk's last block leaves the result where the copy back takes it
+            ba.finish.host = reinterpret_cast<unsigned long long *>(d_result) - 2;
+            ba.finish.ws = reinterpret_cast<unsigned long long *>(d_counters);
+            ba.finish.task_out = reinterpret_cast<unsigned long long *>(d_tasks);
+            ba.finish.ntasks = P.ntasks;
+        }
         ba.mats = reinterpret_cast<const pk::BatchMat *>(scratch + kOffBatchMat);
         ba.devmats = scratch + kOffImage;
         ba.ntasks = P.ntasks;
@@ -174,20 +186,18 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
         ba.abort_flag = reinterpret_cast<unsigned int *>(d_counters + 3);
         if ((e = P.gf.walk(ba, P.grid, P.block, st_)) != cudaSuccess) return failed(cuda_fail(e, "walk kernel launch"));
     }
-    if ((e = reduce_launch(P.arith, reinterpret_cast<uint64_t *>(d_tasks), P.ntasks, d_result, d_counters + 4, st_)) !=
+    if (!fused &&
+        (e = reduce_launch(P.arith, reinterpret_cast<uint64_t *>(d_tasks), P.ntasks, d_result, d_counters + 4, st_)) !=
         cudaSuccess)
         return failed(cuda_fail(e, "reduce kernel launch"));
-    uint64_t host[4];
+    uint64_t host[kOffResult / 8 + 3];   // counters and result: one copy back
     if ((e = cudaMemcpyAsync(host, d_counters, sizeof(host), cudaMemcpyDeviceToHost, st_)) != cudaSuccess)
-        return failed(cuda_fail(e, "cudaMemcpyAsync(counters)"));
-    uint64_t raw[3];
-    if ((e = cudaMemcpyAsync(raw, d_result, sizeof(raw), cudaMemcpyDeviceToHost, st_)) != cudaSuccess)
         return failed(cuda_fail(e, "cudaMemcpyAsync(result)"));
     if ((e = cudaStreamSynchronize(st_)) != cudaSuccess) return failed(cuda_fail(e, "cudaStreamSynchronize"));
     describe(P, out);
     if (host[3]) return failed(fail(PERM_ERR_TIMEOUT, "device-side deadline passed; the walk stopped early"));
     out->zero_skip_frac = zero_skip_fraction(P, host[1]);
-    return finish_raw(P, raw, out);
+    return finish_raw(P, host + kOffResult / 8, out);
 }
 
 }  // namespace

@@ -34,6 +34,11 @@ constexpr double kAutoDDError = 1e-9;
 constexpr int kAutoDDMaxN = 32;
 bool needs_dd(int n, double perm, double abs_term_sum);
 
+// Most task results that the last block of an eliminated walk sums by itself:
+// beyond, it takes longer than the launch of a reduction kernel (one warp adds
+// 64 results a lane at 2,048 tasks, 304 at 9,728).
+constexpr uint64_t kFusedTasks = 2048;
+
 // Host-side failure injection for tests (perm_debug_inject_failures): each
 // call consumes one pending injected failure of `site`, if any, and the
 // caller then behaves as if the call made there had failed.
@@ -83,6 +88,9 @@ struct perm_plan_s {
     int k = 0, c = 0;         // Algorithm 4 split (codegen)
     int k2 = 0;               // codegen: rows [k, k + k2) of x in shared memory, the rest global
     uint64_t chunk_lo = 0, chunk_hi = 0, ntasks = 0;
+    // The walk's last block sums the task results (finish.cuh): eliminated walks
+    // of few tasks, in plans (their workspace counters start and are left cleared).
+    bool fused() const { return use_elim && ntasks <= perm::kFusedTasks && h_res; }
     perm::GenericFns gf;
     perm::CodegenKernel cg;
     void *d_devmat = nullptr;

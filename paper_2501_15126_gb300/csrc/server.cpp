@@ -426,6 +426,7 @@ struct perm_server_s {
                                 st);
         if (e == cudaSuccess) e = cudaMemsetAsync(w->d_counters, 0, 16, st);
         pk::BatchArgs ba;
+        ba.finish = pk::FinishArgs();
         ba.mats = w->d_table;
         ba.devmats = F.d_images;
         ba.ntasks = t;

@@ -25,6 +25,7 @@
 #ifndef PERM_HOST_EMULATION
 #include <cuda_runtime.h>
 
+#include "finish.cuh"
 #include "vm.hpp"
 #endif
 #include "core.cuh"
@@ -595,13 +596,17 @@ __device__ __forceinline__ void vm_task_loop(const BatchArgs &ba, unsigned char 
     }
 }
 
+#ifndef PERM_HOST_EMULATION
 // One warp per block: a program's slots take 10-45 KB of shared memory, and
 // single-warp blocks fill an SM's 227 KB to the last warp that fits.
 template <class Vm>
 __global__ void __launch_bounds__(32, 8) k_walk_vm(BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char vm_smem[];
     vm_task_loop<Vm>(ba, vm_smem);
+    finish_walk<typename Vm::A>(ba.finish);
 }
+
+#endif
 
 }  // namespace pk
 
