@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libperm.so")
 
-SOURCES = ["host.cpp", "api.cpp", "codegen.cpp", "elim.cpp", "batch.cpp", "tune.cpp", "server.cpp", "generic.cu",
+SOURCES = ["host.cpp", "api.cpp", "codegen.cpp", "elim.cpp", "plan_res.cpp", "batch.cpp", "tune.cpp", "server.cpp", "generic.cu",
            "generic_f64.cu", "generic_dd.cu", "generic_r64.cu", "generic_r96.cu", "generic_r128.cu", "generic_r160.cu",
            "generic_r192.cu", "microbench.cu", "noalloc.cu", "checkpoint.cpp", "xshared.cu", "vm_image.cpp", "vm_f64.cu", "vm_dd.cu", "vm_exact.cu"]
 EMBED = ["core.cuh", "devmat.h", "finish.cuh"]

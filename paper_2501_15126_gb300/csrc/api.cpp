@@ -558,14 +558,11 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
     if (P.dd && engine == PERM_ENGINE_XSHARED) return fail(PERM_ERR_ARG, "the x-in-shared-memory baseline is FP64 only");
     P.engine = engine;
     P.words = result_words(P.arith);
+    std::vector<unsigned char> img;   // what the kernel reads (none: a generated kernel)
 
     if (engine == PERM_ENGINE_XSHARED) {
-        std::vector<unsigned char> img;
         build_xshared_image(P, img);
         P.img_bytes = img.size();
-        if ((e = cudaMalloc(&P.d_devmat, img.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc(CSC image)");
-        if ((e = cudaMemcpy(P.d_devmat, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-            return cuda_fail(e, "cudaMemcpy(CSC image)");
         cudaFuncAttributes attr;
         if ((e = xshared_attr(&attr)) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
         P.regs = attr.numRegs;
@@ -577,9 +574,7 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
         P.gf = generic_fns(P.family_nmax(), P.family_kind());
         if (!P.gf.walk) return fail(PERM_ERR_INTERNAL, "no eliminated walk for this arithmetic");
         P.img_bytes = P.vm_bytes;
-        if ((e = cudaMalloc(&P.d_devmat, P.vm_img.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc(program image)");
-        if ((e = cudaMemcpy(P.d_devmat, P.vm_img.data(), P.vm_img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-            return cuda_fail(e, "cudaMemcpy(program image)");
+        img.swap(P.vm_img);
         cudaFuncAttributes attr;
         if ((e = P.gf.attr(&attr)) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
         P.regs = attr.numRegs;
@@ -590,12 +585,8 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
         P.gf = generic_fns(nmax, P.kind());
         if (!P.gf.walk) return fail(PERM_ERR_INTERNAL, "no generic kernel for this size");
         P.nmax = nmax;
-        std::vector<unsigned char> img;
         build_devmat(P.m, P.L, P.img_kind(), nmax, img);
         P.img_bytes = img.size();
-        if ((e = cudaMalloc(&P.d_devmat, img.size())) != cudaSuccess) return cuda_fail(e, "cudaMalloc(devmat)");
-        if ((e = cudaMemcpy(P.d_devmat, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-            return cuda_fail(e, "cudaMemcpy(devmat)");
         cudaFuncAttributes attr;
         if ((e = P.gf.attr(&attr)) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
         P.regs = attr.numRegs;
@@ -627,25 +618,39 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
             if ((e = cudaMalloc(&P.d_xglob, bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc(x global rows)");
         }
     }
+    // one device buffer: image, workspace words, task results; the first two are
+    // staged in pinned memory and go up on the first compute's stream
+    const size_t img_room = (img.size() + 255) & ~(size_t)255;
     const size_t ws_words = kWsTaskOut + (size_t)P.ntasks * P.words;
-    if ((e = cudaMalloc(&P.d_ws, ws_words * 8)) != cudaSuccess) return cuda_fail(e, "cudaMalloc(workspace)");
+    if ((e = plan_res_take(img_room + ws_words * 8, &P.res)) != cudaSuccess) return cuda_fail(e, "plan buffers");
+    P.d_devmat = P.res.dev;
+    P.d_ws = reinterpret_cast<uint64_t *>(P.res.dev + img_room);
+    P.h_res = P.res.host;
+    P.ev0 = P.res.ev0;
+    P.ev1 = P.res.ev1;
+    uint64_t head[kWsTaskOut];
+    std::memset(head, 0, sizeof head);
     if (engine == PERM_ENGINE_GENERIC && !P.direct) {
         pk::BatchMat bm;
         std::memset(&bm, 0, sizeof(bm));
-        bm.task_begin = 0;
-        bm.out_offset = 0;
-        bm.image = 0;
         bm.chunk_lo = P.chunk_lo;
         bm.chunk_hi = P.chunk_hi;
         bm.K = P.K;
         bm.abs_shift = P.abs_shift;
-        if ((e = cudaMemcpy(P.d_ws + kWsBatchMat, &bm, sizeof(bm), cudaMemcpyHostToDevice)) != cudaSuccess)
-            return cuda_fail(e, "cudaMemcpy(batch table)");
+        std::memcpy(head + kWsBatchMat, &bm, sizeof(bm));
     }
-    if ((e = cudaMallocHost(&P.h_res, 8 * 8)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
-    if (P.fused() && (e = cudaMemset(P.d_ws, 0, 8 * 8)) != cudaSuccess) return cuda_fail(e, "cudaMemset(counters)");
-    if ((e = cudaEventCreate(&P.ev0)) != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
-    if ((e = cudaEventCreate(&P.ev1)) != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
+    P.upload_bytes = img_room + sizeof head;
+    P.uploaded = false;
+    if (P.upload_bytes <= kStageBytes) {
+        if (!img.empty()) std::memcpy(P.res.stage(), img.data(), img.size());
+        std::memcpy(P.res.stage() + img_room, head, sizeof head);
+    } else {   // an image beyond the staging area (dense n > 40) goes up now
+        if ((e = cudaMemcpy(P.res.dev, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+            (e = cudaMemcpy(P.d_ws, head, sizeof head, cudaMemcpyHostToDevice)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(nullptr)) != cudaSuccess)
+            return cuda_fail(e, "cudaMemcpy(image)");
+        P.uploaded = true;
+    }
     P.ms_plan += now_ms() - t0 - P.ms_compile;
     return PERM_OK;
 }
@@ -655,6 +660,9 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
 // replayed graph is timed by events around its launch instead.
 perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events) {
     cudaError_t e;
+    if (!P.uploaded &&
+        (e = cudaMemcpyAsync(P.res.dev, P.res.stage(), P.upload_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        return cuda_fail(e, "cudaMemcpyAsync(image)");
     const bool fused = P.fused();   // one launch: counters are clear, the walk writes h_res
     if (!fused && (e = cudaMemsetAsync(P.d_ws, 0, 8 * 8, st)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     uint64_t *task_out = P.d_ws + kWsTaskOut;
@@ -921,12 +929,8 @@ int perm_plan_s::family_nmax() const {
 }
 
 perm_plan_s::~perm_plan_s() {
-    if (d_devmat) cudaFree(d_devmat);
-    if (d_ws) cudaFree(d_ws);
+    perm::plan_res_give(res);
     if (d_xglob) cudaFree(d_xglob);
-    if (h_res) cudaFreeHost(h_res);
-    if (ev0) cudaEventDestroy(ev0);
-    if (ev1) cudaEventDestroy(ev1);
     if (graph) cudaGraphExecDestroy(graph);
     if (cap_stream) cudaStreamDestroy(cap_stream);
     perm::codegen_release(*this);
@@ -1009,6 +1013,7 @@ static perm_status_t compute_one(perm_plan_t plan, void *stream, perm_result_t *
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { out->status = PERM_ERR_CUDA; return cuda_fail(e, "cudaStreamSynchronize"); }
         plan->computes += 1;
+        plan->uploaded = true;
     }
     return plan_finish(*plan, out);
 }

@@ -54,15 +54,24 @@ __device__ __forceinline__ void finish_walk(const FinishArgs &f) {
     __shared__ u64 sh[32 * A::ACC_WORDS];
     if (!last_block(f.ws + 7)) return;
     typename A::Acc acc = A::acc_zero();
-    for (u64 t = threadIdx.x; t < f.ntasks; t += blockDim.x) acc = A::acc_add(acc, acc_load_l2<A>(f.task_out + t * (u64)A::ACC_WORDS));
+    constexpr int kAhead = 8;   // results under way per thread: a load from L2 takes as long as dozens of additions
+    for (u64 t0 = threadIdx.x; t0 < f.ntasks; t0 += (u64)kAhead * blockDim.x) {
+        typename A::Acc a[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const u64 t = t0 + (u64)i * blockDim.x;
+            a[i] = t < f.ntasks ? acc_load_l2<A>(f.task_out + t * (u64)A::ACC_WORDS) : A::acc_zero();
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) acc = A::acc_add(acc, a[i]);
+    }
     acc = block_sum<A>(acc, sh);
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0) {   // (the end of the launch makes these visible to the host)
         f.host[1] = 0;
         f.host[6] = 0;
         A::acc_store(f.host + 2, A::acc_norm(acc));
         f.ws[0] = 0;
         f.ws[7] = 0;
-        __threadfence_system();
     }
 }
 

@@ -12,6 +12,7 @@
 #include "vm.hpp"
 #include "host.hpp"
 #include "kernels.hpp"
+#include "plan_res.hpp"
 
 namespace perm {
 
@@ -99,6 +100,9 @@ struct perm_plan_s {
     size_t xs_bytes() const { return (size_t)k2 * 256 * (arith == 0 ? 8 : 4); }   // per block
     uint64_t *h_res = nullptr;  // pinned copy of d_ws[0..7]
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    perm::PlanRes res;                     // owns d_devmat, d_ws, h_res, ev0, ev1
+    size_t upload_bytes = 0;               // staged image and workspace header, sent with the first compute
+    bool uploaded = false;
     int computes = 0;                      // perm_compute calls so far
     cudaStream_t cap_stream = nullptr;     // stream the graph is captured on
     cudaGraphExec_t graph = nullptr;       // the captured launches (second call on)
@@ -159,7 +163,7 @@ int range_free_cols(const perm_plan_s &P);
 // Plans the eliminated walk of the precompiled kernels and builds its image
 // (P.vm, P.use_elim): full_blocks as in ElimLimits.  vm_rebuild writes the image
 // again for the plan's current arithmetic (a double-double rerun).
-constexpr double kVmFullBlocks = 16384.0;   // single matrices: outer steps that fill the GPU
+constexpr double kVmFullBlocks = 8192.0;   // single matrices: outer steps that fill the GPU
 constexpr double kVmFullBlocksShared = 64.0;   // batch and serving: other matrices fill it
 // Below min_n the chained walk takes less time than the planning.
 constexpr int kVmMinBatch = 9, kVmMinServe = 22;
