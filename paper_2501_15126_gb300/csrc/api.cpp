@@ -214,8 +214,16 @@ static bool exact_fits_int32(const Matrix &m) {
     return true;
 }
 
+void settle_order(perm_plan_s &P) {
+    if (!P.order_pending) return;
+    P.order_pending = false;
+    P.L = choose_layout(P.m, PERM_ORDER_AUTO);
+    P.ops_per_step = cost_per_step(P.L, false);
+    P.ops_per_step_paper = cost_per_step(P.L, true);
+}
+
 perm_status_t plan_prepare(const perm_matrix_t *A, const perm_opts_t *opts_in, perm_plan_s &P, void *storage,
-                           size_t storage_bytes) {
+                           size_t storage_bytes, bool lazy_order) {
     const double t0 = now_ms();
     perm_opts_t opts;
     std::memset(&opts, 0, sizeof(opts));
@@ -250,7 +258,9 @@ perm_status_t plan_prepare(const perm_matrix_t *A, const perm_opts_t *opts_in, p
         P.abs_shift = abs_shift_for(P.m);
         P.dd = opts.precision == PERM_PREC_DD;
     }
-    P.L = choose_layout(P.m, opts.ordering);
+    // (a sub-range's partial sum belongs to the plan's order)
+    P.order_pending = lazy_order && !P.subrange && opts.ordering == PERM_ORDER_AUTO && elim_allowed(P);
+    P.L = choose_layout(P.m, opts.ordering, !P.order_pending);
     P.ops_per_step = cost_per_step(P.L, false);
     P.ops_per_step_paper = cost_per_step(P.L, true);
     if (P.m.is_int) {
@@ -479,7 +489,7 @@ bool vm_rebuild(perm_plan_s &P) {
     return P.vm_bytes <= (size_t)kVmMaxWarpBytes;
 }
 
-bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
+static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
     P.vm = P.use_elim = false;
     adopt_elim(P);
     const int n = P.m.n;
@@ -500,7 +510,7 @@ bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
     ElimLimits lim;
     lim.full_blocks = full_blocks;
     lim.allow_none = lim.tables_only = true;
-    lim.candidates = n <= 20 ? 4 : n <= 23 ? 8 : n <= 26 ? 16 : kNMax;
+    lim.candidates = n <= 20 ? 4 : n <= 25 ? 8 : 12;   // 25 us at n = 16, 100-200 at 28
     for (int width = 5; width >= 3; --width) {
         lim.max_width = width;
         if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;
@@ -514,6 +524,12 @@ bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
         P.vm = P.use_elim = false;
         P.vm_img.clear();
     }
+    return false;
+}
+
+bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
+    if (vm_plan(P, full_blocks, min_n)) return true;
+    settle_order(P);   // the chained walk's
     return false;
 }
 
@@ -555,6 +571,7 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
     if (engine == PERM_ENGINE_GENERIC && n > 48) return fail(PERM_ERR_SIZE, "generic kernels cover n <= 48");
     const int nmax = nmax_bucket(std::min(n, 48));
     if (tiny && engine != PERM_ENGINE_XSHARED) engine = PERM_ENGINE_GENERIC;
+    if (engine != PERM_ENGINE_GENERIC || tiny) settle_order(P);
     if (P.dd && engine == PERM_ENGINE_XSHARED) return fail(PERM_ERR_ARG, "the x-in-shared-memory baseline is FP64 only");
     P.engine = engine;
     P.words = result_words(P.arith);
@@ -912,7 +929,7 @@ static perm_status_t make_dd_plan(perm_plan_s &P) {
     o.ordering = P.L.ordering == PERM_ORDER_SEARCH ? PERM_ORDER_AUTO : P.L.ordering;
     perm_plan_s *D = new (std::nothrow) perm_plan_s();
     if (!D) return fail(PERM_ERR_NOMEM, "out of host memory");
-    perm_status_t st = plan_prepare(&A, &o, *D);
+    perm_status_t st = plan_prepare(&A, &o, *D, nullptr, 0, true);
     if (st == PERM_OK) st = plan_device_setup(*D);
     if (st != PERM_OK) { delete D; return st; }
     P.dd_plan = D;
@@ -946,7 +963,7 @@ perm_status_t perm_plan_create(const perm_matrix_t *A, const perm_opts_t *opts, 
     *out = nullptr;
     perm_plan_s *P = new (std::nothrow) perm_plan_s();
     if (!P) return fail(PERM_ERR_NOMEM, "out of host memory");
-    perm_status_t st = plan_prepare(A, opts, *P);
+    perm_status_t st = plan_prepare(A, opts, *P, nullptr, 0, true);
     if (st == PERM_OK) st = plan_device_setup(*P);
     if (st != PERM_OK) { delete P; return st; }
     *out = P;

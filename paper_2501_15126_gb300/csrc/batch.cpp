@@ -339,7 +339,7 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
         auto work = [&](int t) {
             for (int32_t i = t; i < count; i += nthreads) {
                 plans[i].reset(new perm_plan_s());
-                prep[i] = plan_prepare(&mats[i], &opts, *plans[i]);
+                prep[i] = plan_prepare(&mats[i], &opts, *plans[i], nullptr, 0, true);
                 if (prep[i] == PERM_OK && !plans[i]->zero) vm_prepare(*plans[i], kVmFullBlocksShared, kVmMinBatch);
             }
         };
@@ -382,6 +382,7 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
                 P.dd = true;
                 if (P.vm && !vm_rebuild(P)) {   // too many pair slots: the chained walk
                     P.vm = P.use_elim = false;
+                    settle_order(P);
                     adopt_elim(P);
                 }
                 redo[{P.family_nmax(), P.family_kind()}].add(i, &P);

@@ -419,7 +419,7 @@ double walk_cost_per_step(const Layout &L, bool fp64) {
     return L.n >= 31 ? std::min(dual, cost_per_step_paired(L)) : dual;
 }
 
-Layout choose_layout(const Matrix &m, int ordering_opt) {
+Layout choose_layout(const Matrix &m, int ordering_opt, bool search) {
     int cols[kNMax], rows[kNMax];
     if (ordering_opt == PERM_ORDER_NONE) { order_none(m, cols); return make_layout(m, cols, PERM_ORDER_NONE); }
     if (ordering_opt == PERM_ORDER_DEGREE) { order_degree(m, cols); return make_layout(m, cols, PERM_ORDER_DEGREE); }
@@ -438,7 +438,7 @@ Layout choose_layout(const Matrix &m, int ordering_opt) {
     // FP64 half: 2.15 s -> 1.76 s).  Exact kernels fold runs of rows in 32
     // bits, which the one-chain model does not see (a searched order made the
     // n=48 band's exact walk 7 % slower), so they keep the start order.
-    if (m.n < 22 || m.is_int) return start;
+    if (m.n < 22 || m.is_int || !search) return start;
     for (int p = 0; p < m.n; ++p) cols[p] = start.col_order[p];
     const bool fp64 = true, long_walk = m.n >= 31;
     const double before = order_cost(m, cols, fp64, long_walk);

@@ -93,8 +93,9 @@ double cost_per_step(const Layout &L, bool paper_scheme);
 // even step's flip rebuilds levels j..1 only.
 double cost_per_step_paired(const Layout &L);
 
-// Chooses the ordering (AUTO = cheaper of DEGREE and PAPER under the model).
-Layout choose_layout(const Matrix &m, int ordering_opt);
+// Chooses the ordering (AUTO = cheaper of DEGREE and PAPER under the model, then
+// a search from it for FP64 walks of 2^21 steps and more unless search is false).
+Layout choose_layout(const Matrix &m, int ordering_opt, bool search = true);
 
 // Algorithm 4 with GB300 occupancy; returns k (register rows) and c.
 void partition_alg4(const Layout &L, double gr_ratio, int base_regs, int *k, int *c);

@@ -106,6 +106,7 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     }
     if (!vm) {
         P.vm = P.use_elim = false;
+        settle_order(P);
         adopt_elim(P);
         P.gf = generic_fns(nmax_bucket(n), P.kind());
         if (!P.gf.walk) return failed(fail(PERM_ERR_INTERNAL, "no generic kernel"));
@@ -219,7 +220,7 @@ extern "C" perm_status_t perm_compute_noalloc(const perm_matrix_t *A, const perm
 
     alignas(16) unsigned char dense[kNoAllocMaxN * kNoAllocMaxN * 8];
     perm_plan_s P;   // host bookkeeping only: nothing on the device is allocated through it
-    st = plan_prepare(A, opts, P, dense, sizeof(dense));
+    st = plan_prepare(A, opts, P, dense, sizeof(dense), true);
     if (st != PERM_OK) return failed(st);
     if (P.zero) { describe(P, out); out->status = PERM_OK; return PERM_OK; }
     cudaStream_t st_ = reinterpret_cast<cudaStream_t>(stream);

@@ -78,6 +78,7 @@ struct perm_plan_s {
     uint64_t total = 0;       // 2^(n-1)
     uint64_t g_lo = 0, g_hi = 0;
     bool subrange = false;
+    bool order_pending = false;   // L is the order search's start (settle_order)
     bool zero = false;        // no perfect matching: perm is 0, nothing launches
     bool direct = false;      // tiny n: one thread per Gray index
     double bound = 0.0;
@@ -135,8 +136,12 @@ double now_ms();
 
 // Stages of perm_plan_create / perm_compute, reused by batch and serving.
 // storage: optional caller memory (>= n*n*8 bytes) for the dense copy.
+// lazy_order: a whole FP64 walk's column order is left unsearched (0.2-0.7 ms of
+// host time at n = 22..28) until settle_order, which whatever walks in that
+// order calls: the eliminated walk of a whole range orders its columns itself.
 perm_status_t plan_prepare(const perm_matrix_t *A, const perm_opts_t *opts, perm_plan_s &P,
-                           void *storage = nullptr, size_t storage_bytes = 0);
+                           void *storage = nullptr, size_t storage_bytes = 0, bool lazy_order = false);
+void settle_order(perm_plan_s &P);
 perm_status_t plan_device_setup(perm_plan_s &P);
 perm_status_t plan_launch(perm_plan_s &P, cudaStream_t st, bool record_events = true);
 perm_status_t plan_finish(perm_plan_s &P, perm_result_t *out);
@@ -166,7 +171,7 @@ int range_free_cols(const perm_plan_s &P);
 constexpr double kVmFullBlocks = 8192.0;   // single matrices: outer steps that fill the GPU
 constexpr double kVmFullBlocksShared = 64.0;   // batch and serving: other matrices fill it
 // Below min_n the chained walk takes less time than the planning.
-constexpr int kVmMinBatch = 9, kVmMinServe = 22;
+constexpr int kVmMinBatch = 9, kVmMinServe = 22;   // (a submitter plans alone: 40 us at n = 22)
 bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n);
 bool vm_rebuild(perm_plan_s &P);
 // Task chunks of a matrix that shares a launch with others: outer steps per lane.

@@ -53,7 +53,10 @@ constexpr int kStreams = 2;                   // wave streams; one more (aux) ta
 constexpr uint64_t kSmallShare = 64;          // tasks every active request gets per wave
 constexpr double kWaveSteps = 268435456.0;    // Gray steps per wave (2^28, a few ms): short waves let
                                               // requests that arrive meanwhile start soon
-constexpr int kServeChunkLog2 = 12;           // chunk length target: tasks of 2^17 steps fill short waves
+// Chunk length target of the chained walk: 2^12 steps fill short waves, but a
+// small matrix takes 2^8 and spreads over more warps (n = 18..21: a chunk of 2^12
+// steps took a lane 6 ms).
+int serve_chunk_log2(int n) { return std::max(std::min(12, std::max(8, n - 12)), n - 26); }
 constexpr int kAdmitScan = 256;               // queued requests looked at past a blocked one
 constexpr double kNoSkipAfterMs = 200.0;      // a request blocked this long stops being overtaken
 constexpr size_t kQueueMax = 1 << 20;
@@ -301,7 +304,7 @@ struct perm_server_s {
             if (F.vm) {
                 choose_shared_chunks(P, 20);
             } else {
-                P.K = batch_chunk_log2(P.m.n, F.gf.block_log2, std::max(kServeChunkLog2, P.m.n - 26));
+                P.K = batch_chunk_log2(P.m.n, F.gf.block_log2, serve_chunk_log2(P.m.n));
                 P.chunk_lo = 0;
                 P.chunk_hi = P.total >> P.K;
                 P.ntasks = (P.chunk_hi + 31) / 32;
@@ -532,6 +535,7 @@ struct perm_server_s {
         P.dd = true;
         if (P.vm && (!vm_rebuild(P) || P.vm_img.size() > kVmImageCap)) {   // too many pair slots: the chained walk
             P.vm = P.use_elim = false;
+            settle_order(P);
             adopt_elim(P);
         }
         const int nmax = P.family_nmax(), kind = P.family_kind();
@@ -734,13 +738,15 @@ perm_status_t perm_submit(perm_server_t s, const perm_matrix_t *A, uint64_t *tic
     perm_opts_t po;
     std::memset(&po, 0, sizeof(po));
     po.precision = s->opts.precision;
-    perm_status_t st = plan_prepare(A, &po, *r->P);
+    perm_status_t st = plan_prepare(A, &po, *r->P, nullptr, 0, true);
     if (st != PERM_OK) return st;
     perm_plan_s &P = *r->P;
     // a server with a deadline keeps the chained walk, as a call with one does
-    if (!P.zero && s->opts.timeout_ms == 0 && vm_prepare(P, kVmFullBlocksShared, kVmMinServe) &&
-        P.vm_img.size() > kVmImageCap) {
+    if (P.zero || s->opts.timeout_ms != 0) {
+        settle_order(P);
+    } else if (vm_prepare(P, kVmFullBlocksShared, kVmMinServe) && P.vm_img.size() > kVmImageCap) {
         P.vm = P.use_elim = false;
+        settle_order(P);
         adopt_elim(P);
     }
     r->t_submit = now_ms();
