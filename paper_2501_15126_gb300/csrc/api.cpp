@@ -497,8 +497,8 @@ static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
     const double range = std::log2((double)(P.g_hi - P.g_lo));
     // Where the line lies: chained -> eliminated, single matrices: n=17 p=0.3 FP64
     // 0.228 -> 0.024 ms, n=24 p=0.2 FP64 0.21 -> 0.039 ms and 0/1 0.082 -> 0.020 ms,
-    // n=28 p=0.3 FP64 3.0 -> 1.33 ms, n=23 p=0.25 double-double 0.95 -> 0.13 ms a
-    // call; n=28 p=0.4 0/1, whose rows share too much, stays with the chain (2.2 ms).
+    // n=28 p=0.3 FP64 3.0 -> 1.23 ms, n=23 p=0.25 double-double 0.95 -> 0.13 ms a
+    // call, n=28 p=0.4 0/1 2.2 -> 1.24 ms.
     // The chained walk's time in lane-operations of the whole GPU.  Alone, a walk
     // of fewer than 152 blocks' tasks (eight 32-chunk tasks of 2^8 steps, exact
     // 2^6) leaves SMs idle; an exact chained step takes as long as nine operations
@@ -510,7 +510,9 @@ static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
     ElimLimits lim;
     lim.full_blocks = full_blocks;
     lim.allow_none = lim.tables_only = true;
-    lim.candidates = n <= 20 ? 4 : n <= 25 ? 8 : 12;   // 25 us at n = 16, 100-200 at 28
+    // planning takes 25 us at n = 16 and 200-290 at 28, where all candidates lower the
+    // operations by 7 % on 8 (n=28 p=0.3: 0.87 -> 0.80 ms a permanent)
+    lim.candidates = n <= 20 ? 4 : n <= 25 ? 8 : n;
     for (int width = 5; width >= 3; --width) {
         lim.max_width = width;
         if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;

@@ -23,14 +23,15 @@ struct Sim {
 
 // The order in which the tables of a bucket are multiplied: smallest scope
 // first, then always the table that grows the joint scope least.
-int bucket_order(const uint64_t *scope, const int *idx, int t, int *seq) {
+// (`late`, if given, marks tables to come after all others.)
+int bucket_order(const uint64_t *scope, const int *idx, int t, int *seq, const int *late = nullptr) {
     bool used[2 * kNMax] = {};
     uint64_t u = 0;
     for (int s = 0; s < t; ++s) {
         int best = -1, bk = 1 << 30;
         for (int i = 0; i < t; ++i) {
             if (used[i]) continue;
-            const int key = pc(u | scope[idx[i]]) * 64 + pc(scope[idx[i]]);
+            const int key = pc(u | scope[idx[i]]) * 64 + pc(scope[idx[i]]) + (late && late[idx[i]] >= 0 ? 1 << 16 : 0);
             if (key < bk) { bk = key; best = i; }
         }
         used[best] = true;
@@ -277,7 +278,25 @@ void build_tables(const Matrix &m, ElimPlan &E, const int *order, int k) {
         for (int i = 0; i < nitems; ++i)
             if (item_scope[i] & b) idx[t++] = i;
         if (!t) continue;
+        // FP64: the order with all rows first where that is cheaper, an entry of a
+        // product with a summed-out table (a magnitude too) counted as two
         bucket_order(item_scope, idx, t, seq);
+        if (!m.is_int) {
+            auto cost = [&](const int *order) {
+                uint64_t u = item_scope[order[0]];
+                bool summed = item_tab[order[0]] >= 0;
+                double c = 0.0;
+                for (int s = 1; s < t; ++s) {
+                    u |= item_scope[order[s]];
+                    summed |= item_tab[order[s]] >= 0;
+                    c += (double)(1ull << pc(u)) * (summed ? 2.0 : 1.0);
+                }
+                return c;
+            };
+            int rows_first[2 * kNMax];
+            bucket_order(item_scope, idx, t, rows_first, item_tab);
+            if (cost(rows_first) < cost(seq)) std::copy(rows_first, rows_first + t, seq);
+        }
         // a row becomes a table just before it is multiplied, and up to three more of
         // the bucket's rows of the same small size with it (one instruction)
         auto make_row = [&](int it) {

@@ -78,24 +78,48 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
         for (const ElimTableOp &op : tops)
             summed[op.dst] = op.kind == kTabSum || op.kind == kTabSub || (op.kind == kTabMul && (summed[op.a] || summed[op.b]));
     for (int i = 0; i < n; ++i) slot[i] = i;
-    auto take = [&](int t) { slot[t] = (is_ring(t) ? extra : plain).take(size_of(t)); };
+    // A bucket's running product keeps one range from its first row on: the range
+    // is as large as the product will become, new columns take the upper index
+    // bits, and the walk multiplies blocks of entries from the top down, so that
+    // every product overwrites its own operand last.
+    std::vector<int> room(ntab, 0);
+    std::vector<std::vector<int>> bits(ntab);   // a table's columns (elimination places) by index bit
+    auto grown = [&](int t) {
+        int size = size_of(t);
+        for (int u = t; last[u] >= 0 && last[u] < end;) {
+            const ElimTableOp &op = tops[last[u]];
+            if (op.kind != kTabMul || op.a != u || op.b == u || is_ring(op.dst) != is_ring(t)) break;
+            u = op.dst;
+            size = size_of(u);
+        }
+        return size;
+    };
+    auto take = [&](int t, int size) {
+        room[t] = size;
+        slot[t] = (is_ring(t) ? extra : plain).take(size);
+    };
+    auto own_bits = [&](int t) {
+        for (uint64_t x = E.tables[t].scope; x; x &= x - 1) bits[t].push_back(__builtin_ctzll(x));
+    };
     auto take_mag = [&](int t) {
         if (summed[t]) mag[t] = extra.take(size_of(t));
     };
     auto give = [&](int t, int q, bool keep_slot) {
         if (t < n || last[t] != q) return;
-        if (!keep_slot) (is_ring(t) ? extra : plain).give(slot[t], size_of(t));
+        if (!keep_slot) (is_ring(t) ? extra : plain).give(slot[t], room[t]);
         if (summed[t]) extra.give(mag[t], size_of(t));
     };
     auto ref = [&](int t) { return (unsigned short)(is_ring(t) ? slot[t] | (int)pk::kVmRingSlot : slot[t]); };
     auto mref = [&](int t) { return (unsigned short)(mag[t] >= 0 ? mag[t] : (int)pk::kVmNoMag); };
-    // strides of operand t over the columns of `scope` (index bits of the result)
-    auto step = [&](int t, uint64_t b, int unit) {
-        return (unsigned short)((E.tables[t].scope & b) ? unit << __builtin_popcountll(E.tables[t].scope & (b - 1)) : 0);
+    // the stride of column place q in table t, and operand t's strides over the
+    // result's index bits
+    auto step = [&](int t, int q, int unit) {
+        for (size_t k = 0; k < bits[t].size(); ++k)
+            if (bits[t][k] == q) return (unsigned short)(unit << k);
+        return (unsigned short)0;
     };
-    auto strides = [&](int t, uint64_t scope, int unit, unsigned short *s) {
-        int k = 0;
-        for (uint64_t x = scope; x; x &= x - 1, ++k) s[k] = step(t, x & (~x + 1), unit);
+    auto strides = [&](int t, int dst, int unit, unsigned short *s) {
+        for (size_t k = 0; k < bits[dst].size(); ++k) s[k] = step(t, bits[dst][k], unit);
     };
     const int slot_bytes = img == kImgDD ? 512 : 256;
     std::vector<pk::VmIns> prog;
@@ -109,7 +133,8 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
         if (w > pk::kVmBits) return false;
         I.w = (unsigned char)w;
         if (op.kind == kTabRow) {
-            take(op.dst);
+            take(op.dst, grown(op.dst));
+            own_bits(op.dst);
             if (w > pk::kVmRowBits) {
                 I.kind = pk::kVmBigRow;
                 I.dst = (unsigned short)slot[op.dst];
@@ -134,12 +159,21 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
             for (uint64_t x = scope; x; x &= x - 1) row.lit[k++] = (unsigned short)lit(op.a, E.low[__builtin_ctzll(x)]);
             continue;
         }
-        const uint64_t b = 1ull << op.col;
-        // an operand over the result's own columns may be overwritten entry by entry
-        const bool in_place = op.kind == kTabMul && op.a >= n && last[op.a] == q && E.tables[op.a].scope == scope &&
-                              is_ring(op.a) == is_ring(op.dst) && op.a != op.b;
-        if (in_place) slot[op.dst] = slot[op.a];
-        else take(op.dst);
+        const bool in_place = op.kind == kTabMul && op.a >= n && last[op.a] == q && op.a != op.b &&
+                              is_ring(op.a) == is_ring(op.dst) && room[op.a] >= size_of(op.dst);
+        if (op.kind == kTabMul) {   // A's columns first: what is left of the index is new
+            bits[op.dst] = bits[op.a];
+            for (int k : bits[op.b])
+                if (std::find(bits[op.dst].begin(), bits[op.dst].end(), k) == bits[op.dst].end()) bits[op.dst].push_back(k);
+        } else {
+            own_bits(op.dst);
+        }
+        if (in_place) {
+            slot[op.dst] = slot[op.a];
+            room[op.dst] = room[op.a];
+        } else {
+            take(op.dst, op.kind == kTabMul ? grown(op.dst) : size_of(op.dst));
+        }
         take_mag(op.dst);
         I.kind = (unsigned char)(op.kind == kTabSum   ? pk::kVmSum
                                  : op.kind == kTabSub ? pk::kVmSub
@@ -152,10 +186,10 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
         I.t.fa = mref(op.a);
         I.t.fb = mref(op.b);
         const int unit = is_ring(op.dst) ? 1 : slot_bytes;
-        strides(op.a, scope, unit, I.t.sa);
-        strides(op.b, scope, unit, I.t.sb);
-        I.t.ea = step(op.a, b, unit);
-        I.t.eb = step(op.b, b, unit);
+        strides(op.a, op.dst, unit, I.t.sa);
+        strides(op.b, op.dst, unit, I.t.sb);
+        I.t.ea = step(op.a, op.col, unit);
+        I.t.eb = step(op.b, op.col, unit);
         give(op.a, q, in_place);
         if (op.b != op.a) give(op.b, q, false);
         prog.push_back(I);

@@ -11,11 +11,13 @@
 // hide one another's latency.  The value slots of a warp (10-40 KB) set how many
 // warps an SM holds, so there is one value per lane and slot.
 //
-// Measured (n=28 p=0.3 FP64, 2.96 operations per Gray step, 5 warps per SM): FP64
-// pipe 58 % active, 1.32 ms; scalar instructions in bundles of four, one value
-// per slot, 56 % at 6 warps; two values per lane and slot (half the decoding, half
-// the warps) 1.86 ms; tables of 2^4 entries (7 warps, 24 % more operations) 1.50 ms,
-// of 2^6 (4 warps, 15 % fewer) 1.30 ms, but 3.1 against 2.7 ms at p=0.4.
+// Measured (n=28 p=0.3 FP64, 2^27 Gray steps): 1.23 ms, 6 warps per SM; with a
+// range of slots per partial product, 10 % more slots and 5 warps, 1.33 ms at
+// 58 % FP64-pipe activity.  Taken back: scalar instructions in bundles of four, one
+// value per slot, 1.24 ms with 9 % fewer operations (56 % of the pipe); two values
+// per lane and slot (half the decoding, half the warps) 1.86 ms; tables of 2^4
+// entries (7 warps, 24 % more operations) 1.50 ms, of 2^6 (4 warps, 15 % fewer)
+// 1.30 ms, but 3.1 against 2.7 ms at p=0.4.
 //
 // Each warp has its own shared-memory region: the image, then the value slots
 // (slot-major, one word per lane: conflict-free).  Slots belong to one lane,
@@ -196,7 +198,7 @@ struct VmExact {
     __device__ __forceinline__ void ring_table(int kind, int w, unsigned dst, unsigned a, unsigned b, const int *sa,
                                                const int *sb, int ea, int eb) {
 #pragma unroll 1
-        for (int e = 0; e < (1 << w); ++e) {
+        for (int e = (1 << w) - 1; e >= 0; --e) {   // (from the top down: vm_blocks)
             int oa = 0, ob = 0;
 #pragma unroll
             for (int k = 0; k < kVmBits; ++k)
@@ -326,20 +328,20 @@ __device__ __forceinline__ void vm_rows(Vm &vm, int rows, const unsigned (&f)[kV
         }
 }
 
-// Blocks of 2^NB entries over all index bits of a table instruction.
+// Blocks of 2^NB entries over all index bits of a table instruction, from the
+// top down: a result may share its lower part with its first operand (vm_image.cpp).
 template <class Vm, int KIND, int NB>
 __device__ __forceinline__ void vm_blocks(Vm &vm, int w, VmAddr d, VmAddr fd, const VmTab &ta, const VmTab &tb,
                                           const int *sa, const int *sb, int ea, int eb) {
 #pragma unroll 1
-    for (int o = 0; o < (1 << (w - NB)); ++o) {
+    for (int o = (1 << (w - NB)) - 1; o >= 0; --o) {
         VmAddr a = ta.v, b = tb.v;
 #pragma unroll
         for (int k = 0; k + NB < kVmBits; ++k)
             if ((o >> k) & 1) { a += sa[k + NB]; b += sb[k + NB]; }
-        if constexpr (KIND == kVmMul) vm_mul_block<Vm, NB>(d, a, b, sa, sb);
-        else vm_mag_block<Vm, KIND, NB>(vm, d, fd, a, b, ta, tb, sa, sb, ea, eb);
-        d += Vm::kSlot << NB;
-        fd += 128 << NB;
+        const VmAddr e = d + o * (Vm::kSlot << NB);
+        if constexpr (KIND == kVmMul) vm_mul_block<Vm, NB>(e, a, b, sa, sb);
+        else vm_mag_block<Vm, KIND, NB>(vm, e, fd + o * (128 << NB), a, b, ta, tb, sa, sb, ea, eb);
     }
 }
 
