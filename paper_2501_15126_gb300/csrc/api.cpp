@@ -593,7 +593,7 @@ perm_status_t plan_device_setup(perm_plan_s &P) {
         P.gf = generic_fns(P.family_nmax(), P.family_kind());
         if (!P.gf.walk) return fail(PERM_ERR_INTERNAL, "no eliminated walk for this arithmetic");
         P.img_bytes = P.vm_bytes;
-        img.swap(P.vm_img);
+        img.assign(P.vm_img.begin(), P.vm_img.end());
         cudaFuncAttributes attr;
         if ((e = P.gf.attr(&attr)) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
         P.regs = attr.numRegs;

@@ -363,7 +363,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
     // candidates: the free columns by ascending size
     int cand[kNMax], nc = 0;
     for (int p = 0; p < free_n; ++p) cand[nc++] = col_order[p];
-    std::stable_sort(cand, cand + nc, [&](int a, int b) { return pc(m.colmask[a]) < pc(m.colmask[b]); });
+    insertion_sort(cand, cand + nc, [&](int a, int b) { return pc(m.colmask[a]) < pc(m.colmask[b]); });
     // Greedy growth of the low set: the column that lowers the modelled time
     // most.  time = (program + the outer flips' updates + loop) x outer steps,
     // where fewer steps than fill the GPU take as long as those.

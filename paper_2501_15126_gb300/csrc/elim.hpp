@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <memory_resource>
 #include <string>
 #include <vector>
 
@@ -53,22 +54,33 @@ struct ElimTableOp {
     int col;           // sum, sub: the column's place in the elimination order
 };
 
+// (`mem` is where a plan and its image keep their vectors: the heap, or the stack
+// of the allocation-free call.)
 struct ElimPlan {
+    explicit ElimPlan(std::pmr::memory_resource *mem = std::pmr::new_delete_resource())
+        : ops(mem), bound(mem), tables(mem), tops(mem), factors(mem) {}
     int n = 0, k = 0, h = 0;          // k low columns summed out, h outer columns walked
     int low[kNMax] = {};              // low columns in elimination order (original indices)
     int outer[kNMax] = {};            // outer column at Gray position p (original index)
     int last = 0;                     // the column that never flips
     int exp2[kNMax] = {};             // FP64: row i is walked as x_i 2^-exp2[i] (elim_row_bits)
     int scale = 0;                    // FP64: sum of exp2: the walk's sum times 2^scale is the true one
-    std::vector<ElimOp> ops;
+    std::pmr::vector<ElimOp> ops;
     int result = 0;                   // the value that holds the step's signed sum
-    std::vector<double> bound;        // exact: a bound of each value's magnitude (n + ops entries)
-    std::vector<ElimTable> tables;    // 0..n-1: x
-    std::vector<ElimTableOp> tops;
-    std::vector<int> factors;         // the step's sum is the product of these single values
+    std::pmr::vector<double> bound;        // exact: a bound of each value's magnitude (n + ops entries)
+    std::pmr::vector<ElimTable> tables;    // 0..n-1: x
+    std::pmr::vector<ElimTableOp> tops;
+    std::pmr::vector<int> factors;         // the step's sum is the product of these single values
     double table_ops = 0.0;           // operations of the table program
     double ops_per_step = 0.0;        // counted operations per Gray step, flips and accumulation included
 };
+
+// Stable, in place (std::stable_sort takes its scratch from the heap).
+template <class It, class Less>
+void insertion_sort(It b, It e, Less less) {
+    for (It i = b; i != e; ++i)
+        for (It j = i; j != b && less(*j, *(j - 1)); --j) std::swap(*j, *(j - 1));
+}
 
 struct ElimLimits {
     int max_width = 5;                // tables of at most 2^max_width entries while a column is summed out

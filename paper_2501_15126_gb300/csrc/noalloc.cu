@@ -19,7 +19,9 @@
 // work overlaps (on different streams or threads) race on it.
 #include <algorithm>
 #include <cstring>
+#include <memory_resource>
 #include <mutex>
+#include <new>
 
 #include <cuda_runtime.h>
 
@@ -36,6 +38,7 @@ constexpr size_t kOffBatchMat = 192;              // one pk::BatchMat
 constexpr size_t kOffImage = 256;                 // the matrix image (<= 20480 bytes)
 constexpr size_t kImageBytes = 20480;
 constexpr size_t kOffTasks = kOffImage + kImageBytes;   // per-task partial sums
+constexpr size_t kPlannerBytes = 128 * 1024;      // the eliminated walk's plan and program, on the stack
 constexpr int kMaxDevices = 64;
 static_assert(sizeof(pk::BatchMat) <= kOffImage - kOffBatchMat, "task table entry");
 // (finish.cuh writes words 1..6 from two words before the result)
@@ -96,7 +99,11 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     int bps = 0;
     size_t img_bytes = 0;
     // the eliminated walk where its image and task results fit the array
-    bool vm = n > 8 && vm_prepare(P, kVmFullBlocks, 9) && P.vm_img.size() <= kImageBytes;
+    bool vm = false;
+    try {
+        vm = n > 8 && vm_prepare(P, kVmFullBlocks, 9) && P.vm_img.size() <= kImageBytes;
+    } catch (const std::bad_alloc &) {   // the planner's stack is full: the chained walk
+    }
     if (vm) {
         P.gf = generic_fns(P.family_nmax(), P.family_kind());
         if (!P.gf.walk) return failed(fail(PERM_ERR_INTERNAL, "no generic kernel"));
@@ -219,7 +226,10 @@ extern "C" perm_status_t perm_compute_noalloc(const perm_matrix_t *A, const perm
     if (st != PERM_OK) return failed(st);
 
     alignas(16) unsigned char dense[kNoAllocMaxN * kNoAllocMaxN * 8];
-    perm_plan_s P;   // host bookkeeping only: nothing on the device is allocated through it
+    // the planner's vectors live on the stack too
+    alignas(16) unsigned char planner[kPlannerBytes];
+    std::pmr::monotonic_buffer_resource mem(planner, sizeof(planner), std::pmr::null_memory_resource());
+    perm_plan_s P(&mem);   // host bookkeeping only: nothing on the device is allocated through it
     st = plan_prepare(A, opts, P, dense, sizeof(dense), true);
     if (st != PERM_OK) return failed(st);
     if (P.zero) { describe(P, out); out->status = PERM_OK; return PERM_OK; }

@@ -49,6 +49,7 @@ bool debug_fail(int site);
 }  // namespace perm
 
 struct perm_plan_s {
+    explicit perm_plan_s(std::pmr::memory_resource *mem = std::pmr::new_delete_resource()) : elim(mem), vm_img(mem) {}
     perm::Matrix m;
     perm::Layout L;
     perm_opts_t opts{};
@@ -67,7 +68,7 @@ struct perm_plan_s {
     perm::ElimPlan elim;
     int val_shift = 0;        // FP64: the walk's sum is the true one times 2^-val_shift
     bool vm = false;          // generic engine: the eliminated walk from a program image (vm.h)
-    std::vector<unsigned char> vm_img;
+    std::pmr::vector<unsigned char> vm_img;
     size_t vm_bytes = 0;      // per-warp shared memory: the image and its value slots
     // kernel family of the generic engine: an NMAX bucket of the chained walk, or
     // the eliminated walk's shared-memory class

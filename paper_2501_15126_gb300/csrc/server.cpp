@@ -321,7 +321,7 @@ struct perm_server_s {
             r->out_offset = off;
             // the image goes up on the aux stream; every wave waits for the uploads made so far
             std::vector<unsigned char> img;
-            if (F.vm) img.swap(P.vm_img);
+            if (F.vm) img.assign(P.vm_img.begin(), P.vm_img.end());
             else build_devmat(P.m, P.L, F.img, F.nmax, img);
             r->slot_bytes = F.vm ? P.vm_bytes : img.size();
             const cudaError_t e = debug_fail(kSiteUpload) ? cudaErrorInvalidValue

@@ -21,7 +21,7 @@ size_t vm_slot_area(int img, int limbs, int nslots, int nextra);
 // Writes the program image of a planned matrix; img is kImgF64, kImgInt or
 // kImgDD, limbs the exact ring (0 otherwise).  False when the program needs
 // more than `max_slots` slots.
-bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_slots, std::vector<unsigned char> &out);
+bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_slots, std::pmr::vector<unsigned char> &out);
 
 // The kernels of one arithmetic (kind as in generic_fns).
 GenericFns vm_fns(int kind);

@@ -14,7 +14,8 @@ size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 // Consecutive slots for tables, first fit.
 struct SlotRanges {
-    std::vector<char> used;
+    std::pmr::vector<char> used;
+    explicit SlotRanges(std::pmr::memory_resource *mem) : used(mem) {}
     int top = 0;
     int take(int count) {
         int run = 0;
@@ -43,15 +44,19 @@ size_t vm_slot_area(int img, int limbs, int nslots, int nextra) {
     return 32 * (lane * (size_t)nslots + extra * (size_t)nextra);
 }
 
-bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_slots, std::vector<unsigned char> &out) {
+bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_slots, std::pmr::vector<unsigned char> &out) {
+    // working vectors on the stack, beyond that where the image is
+    alignas(16) unsigned char work[48 * 1024];
+    std::pmr::monotonic_buffer_resource local(work, sizeof(work), out.get_allocator().resource());
+    std::pmr::memory_resource *mem = &local;
     const int n = m.n;
     const bool exact = img == kImgInt;
     const int ntab = (int)E.tables.size();
-    std::vector<ElimTableOp> tops = E.tops;
+    const std::pmr::vector<ElimTableOp> &tops = E.tops;
     // literals: the entries that the program and the flips add; literal 0 pads
     int lit_of[kNMax][kNMax];
     std::memset(lit_of, -1, sizeof lit_of);
-    std::vector<std::pair<int, int>> lits(1, {-1, -1});
+    std::pmr::vector<std::pair<int, int>> lits(1, {-1, -1}, mem);
     auto lit = [&](int r, int c) {
         int &l = lit_of[r][c];
         if (l >= 0) return l;
@@ -61,7 +66,7 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     // ring tables: 64-bit slots hold what their bound allows (everything, modulo 2^64, in a 64-bit ring)
     auto is_ring = [&](int t) { return exact && limbs > 2 && !(E.tables[t].bound < 9.2e18); };
     auto size_of = [&](int t) { return 1 << __builtin_popcountll(E.tables[t].scope); };
-    std::vector<int> last(ntab, -1), slot(ntab, -1);
+    std::pmr::vector<int> last(ntab, -1, mem), slot(ntab, -1, mem);
     for (int q = 0; q < (int)tops.size(); ++q) {
         if (tops[q].kind != kTabRow) last[tops[q].a] = last[tops[q].b] = q;
     }
@@ -69,11 +74,11 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     for (int f : E.factors) last[f] = end;
     // `extra` holds ring tables (exact) or the magnitudes of tables in which a
     // column has been summed out (FP64)
-    SlotRanges plain, extra;
+    SlotRanges plain(mem), extra(mem);
     plain.used.assign(n + 1, 1);   // x, padding
     plain.top = n + 1;
-    std::vector<int> mag(ntab, -1);
-    std::vector<char> summed(ntab, 0);
+    std::pmr::vector<int> mag(ntab, -1, mem);
+    std::pmr::vector<char> summed(ntab, 0, mem);
     if (!exact)
         for (const ElimTableOp &op : tops)
             summed[op.dst] = op.kind == kTabSum || op.kind == kTabSub || (op.kind == kTabMul && (summed[op.a] || summed[op.b]));
@@ -82,8 +87,10 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     // is as large as the product will become, new columns take the upper index
     // bits, and the walk multiplies blocks of entries from the top down, so that
     // every product overwrites its own operand last.
-    std::vector<int> room(ntab, 0);
-    std::vector<std::vector<int>> bits(ntab);   // a table's columns (elimination places) by index bit
+    struct Bits { int count = 0, at[pk::kVmBits] = {}; };
+    std::pmr::vector<int> room(ntab, 0, mem);
+    std::pmr::vector<Bits> bits(ntab, Bits(), mem);   // a table's columns (elimination places) by index bit
+    auto has = [](const Bits &b, int col) { return std::find(b.at, b.at + b.count, col) != b.at + b.count; };
     auto grown = [&](int t) {
         int size = size_of(t);
         for (int u = t; last[u] >= 0 && last[u] < end;) {
@@ -99,7 +106,7 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
         slot[t] = (is_ring(t) ? extra : plain).take(size);
     };
     auto own_bits = [&](int t) {
-        for (uint64_t x = E.tables[t].scope; x; x &= x - 1) bits[t].push_back(__builtin_ctzll(x));
+        for (uint64_t x = E.tables[t].scope; x; x &= x - 1) bits[t].at[bits[t].count++] = __builtin_ctzll(x);
     };
     auto take_mag = [&](int t) {
         if (summed[t]) mag[t] = extra.take(size_of(t));
@@ -114,15 +121,15 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     // the stride of column place q in table t, and operand t's strides over the
     // result's index bits
     auto step = [&](int t, int q, int unit) {
-        for (size_t k = 0; k < bits[t].size(); ++k)
-            if (bits[t][k] == q) return (unsigned short)(unit << k);
+        for (int k = 0; k < bits[t].count; ++k)
+            if (bits[t].at[k] == q) return (unsigned short)(unit << k);
         return (unsigned short)0;
     };
     auto strides = [&](int t, int dst, int unit, unsigned short *s) {
-        for (size_t k = 0; k < bits[dst].size(); ++k) s[k] = step(t, bits[dst][k], unit);
+        for (int k = 0; k < bits[dst].count; ++k) s[k] = step(t, bits[dst].at[k], unit);
     };
     const int slot_bytes = img == kImgDD ? 512 : 256;
-    std::vector<pk::VmIns> prog;
+    std::pmr::vector<pk::VmIns> prog(mem);
     prog.reserve(tops.size() + 4);
     for (int q = 0; q < end; ++q) {
         const ElimTableOp &op = tops[q];
@@ -162,9 +169,9 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
         const bool in_place = op.kind == kTabMul && op.a >= n && last[op.a] == q && op.a != op.b &&
                               is_ring(op.a) == is_ring(op.dst) && room[op.a] >= size_of(op.dst);
         if (op.kind == kTabMul) {   // A's columns first: what is left of the index is new
-            bits[op.dst] = bits[op.a];
-            for (int k : bits[op.b])
-                if (std::find(bits[op.dst].begin(), bits[op.dst].end(), k) == bits[op.dst].end()) bits[op.dst].push_back(k);
+            Bits &d = bits[op.dst] = bits[op.a];
+            for (int k = 0; k < bits[op.b].count; ++k)
+                if (!has(d, bits[op.b].at[k])) d.at[d.count++] = bits[op.b].at[k];
         } else {
             own_bits(op.dst);
         }
@@ -196,10 +203,10 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     }
     // the step's sum: the product of the single factors, the exact ones that fit
     // 64 bits first (by bound, in runs whose product still fits), ring ones one by one
-    std::vector<int> plain_f, ring_f;
+    std::pmr::vector<int> plain_f(mem), ring_f(mem);
     for (int f : E.factors) (is_ring(f) ? ring_f : plain_f).push_back(f);
     if (exact)
-        std::stable_sort(plain_f.begin(), plain_f.end(), [&](int a, int b) { return E.tables[a].bound < E.tables[b].bound; });
+        insertion_sort(plain_f.begin(), plain_f.end(), [&](int a, int b) { return E.tables[a].bound < E.tables[b].bound; });
     const bool narrow = exact && limbs > 2;
     bool any = false;
     unsigned short acc = 0, facc = (unsigned short)pk::kVmNoMag;
@@ -265,7 +272,7 @@ bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_sl
     }
     if (plain.top + extra.top > max_slots) return false;
 
-    std::vector<unsigned short> flipptr(E.h + 1, 0), flip;   // bundles of four (slot, literal) pairs
+    std::pmr::vector<unsigned short> flipptr(E.h + 1, 0, mem), flip(mem);   // bundles of four (slot, literal) pairs
     for (int p = 0; p < E.h; ++p) {
         flipptr[p] = (unsigned short)(flip.size() / 8);
         int cnt = 0;
