@@ -941,10 +941,13 @@ static perm_status_t make_dd_plan(perm_plan_s &P) {
 }  // namespace perm
 
 // Shared-memory classes of the eliminated walk: a launch takes the largest
-// program's region for every warp, so small programs keep to themselves.
+// program's region for every warp, so small programs keep to themselves.  A 500-
+// matrix batch takes 47.5 ms with two lines (20 and 44 KB), where one 44 KB program
+// holds all the 30 KB ones of its class to 5 warps, and 43.5 ms with these four.
 int perm_plan_s::family_nmax() const {
     if (!vm) return perm::nmax_bucket(m.n);
-    return vm_bytes <= 20 * 1024 ? 1 : vm_bytes <= 44 * 1024 ? 2 : 3;
+    const size_t kb = (vm_bytes + 1023) / 1024;   // 10, 8, 6, 5 and fewer warps an SM
+    return kb <= 21 ? 1 : kb <= 27 ? 2 : kb <= 36 ? 3 : kb <= 44 ? 4 : perm::kVmClasses;
 }
 
 perm_plan_s::~perm_plan_s() {

@@ -40,6 +40,9 @@ bool needs_dd(int n, double perm, double abs_term_sum);
 // 64 results a lane at 2,048 tasks, 304 at 9,728).
 constexpr uint64_t kFusedTasks = 2048;
 
+// Shared-memory classes of the eliminated walk (perm_plan_s::family_nmax: 1..kVmClasses).
+constexpr int kVmClasses = 5;
+
 // Host-side failure injection for tests (perm_debug_inject_failures): each
 // call consumes one pending injected failure of `site`, if any, and the
 // caller then behaves as if the call made there had failed.

@@ -192,7 +192,12 @@ struct perm_server_s {
     double t_first = 0.0, t_last = 0.0;
     perm_status_t init_status = PERM_OK;
 
-    // chained walk: 16, 32, 48 -> 0..41; the eliminated walk's classes 1..3 after them
+    // chained walk: 16, 32, 48 -> 0..41; the eliminated walk's classes after them
+    // (a family holds image slots and a result pool: three shared-memory classes do)
+    static int family_nmax(const perm_plan_s &P) {
+        const int c = P.family_nmax();
+        return !P.vm ? c : c <= 1 ? 1 : c < kVmClasses ? 2 : 3;
+    }
     static int family_index(int nmax, int kind) { return (nmax < 16 ? nmax + 2 : nmax / 16 - 1) * 14 + kind; }
 
     perm_status_t init_device() {   // on the creating thread, with `device` current
@@ -538,7 +543,7 @@ struct perm_server_s {
             settle_order(P);
             adopt_elim(P);
         }
-        const int nmax = P.family_nmax(), kind = P.family_kind();
+        const int nmax = family_nmax(P), kind = P.family_kind();
         r->family = family_index(nmax, kind);
         r->slot = -1;
         r->ntasks = r->next_task = r->done_tasks = 0;
@@ -766,8 +771,8 @@ perm_status_t perm_submit(perm_server_t s, const perm_matrix_t *A, uint64_t *tic
         return PERM_OK;
     }
     if (P.m.n > 8 && P.m.n <= 48) {
-        raw->family = perm_server_s::family_index(P.family_nmax(), P.family_kind());
-        st = s->ensure_family(raw->family, P.family_nmax(), P.family_kind());
+        raw->family = perm_server_s::family_index(perm_server_s::family_nmax(P), P.family_kind());
+        st = s->ensure_family(raw->family, perm_server_s::family_nmax(P), P.family_kind());
         if (st != PERM_OK) { s->all.erase(raw->ticket); return st; }
     }
     s->queue.push_back(raw);
