@@ -235,9 +235,11 @@ perm_status_t perm_plan_create(const perm_matrix_t *A, const perm_opts_t *opts, 
 
 /* Runs the Gray-code walk of a plan on `stream` and fills *out.  The plan's
    device buffers are reused; two perm_compute calls on one plan must not
-   overlap.  From the second call on, the plan's launches (workspace reset,
-   walk, reduction, result copy) are captured once into a CUDA graph and
-   replayed with one launch (unless PERM_FLAG_NO_GRAPH).
+   overlap.  Walks of up to 2,048 tasks are one launch, whose last block
+   reduces the task results and writes the pinned result words; others are
+   captured from the second call on (workspace reset, walk, reduction, result
+   copy) into a CUDA graph and replayed with one launch (unless
+   PERM_FLAG_NO_GRAPH).
    Errors: ARG, CUDA, INTERNAL. */
 perm_status_t perm_compute(perm_plan_t plan, void *stream, perm_result_t *out);
 

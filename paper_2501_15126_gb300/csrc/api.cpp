@@ -511,8 +511,9 @@ static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
     lim.full_blocks = full_blocks;
     lim.allow_none = lim.tables_only = true;
     // planning takes 25 us at n = 16 and 200-290 at 28, where all candidates lower the
-    // operations by 7 % on 8 (n=28 p=0.3: 0.87 -> 0.80 ms a permanent)
-    lim.candidates = n <= 20 ? 4 : n <= 25 ? 8 : n;
+    // operations by 7 % on 8 (n=28 p=0.3: 0.87 -> 0.80 ms a permanent); a served
+    // request is planned by its submitter, where four cost half of eight
+    lim.candidates = n <= 20 || min_n == kVmMinServe ? 4 : n <= 25 ? 8 : n;
     for (int width = 5; width >= 3; --width) {
         lim.max_width = width;
         if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;

@@ -192,12 +192,9 @@ struct perm_server_s {
     double t_first = 0.0, t_last = 0.0;
     perm_status_t init_status = PERM_OK;
 
-    // chained walk: 16, 32, 48 -> 0..41; the eliminated walk's classes after them
-    // (a family holds image slots and a result pool: three shared-memory classes do)
-    static int family_nmax(const perm_plan_s &P) {
-        const int c = P.family_nmax();
-        return !P.vm ? c : c <= 1 ? 1 : c < kVmClasses ? 2 : 3;
-    }
+    // chained walk: 16, 32, 48 -> 0..41; the eliminated walk after them
+    // (a family has image slots, a result pool and waves of its own: one shared-memory class)
+    static int family_nmax(const perm_plan_s &P) { return P.vm ? 1 : P.family_nmax(); }
     static int family_index(int nmax, int kind) { return (nmax < 16 ? nmax + 2 : nmax / 16 - 1) * 14 + kind; }
 
     perm_status_t init_device() {   // on the creating thread, with `device` current
@@ -221,7 +218,7 @@ struct perm_server_s {
             if ((e = cudaMallocHost(&f.h_res, 32 * (size_t)maxn)) != cudaSuccess) return cuda_fail(e, "pinned");
             if ((e = cudaMalloc(&f.d_res, 32 * (size_t)maxn)) != cudaSuccess) return cuda_fail(e, "res");
         }
-        fam.resize(84);
+        fam.resize(56);
         return PERM_OK;
     }
 
