@@ -396,7 +396,8 @@ def run_ours(args):
                 "note": "perm_plan_create + perm_compute + perm_plan_destroy from a host CSR matrix; the matrix "
                         "reaches the GPU inside the generated kernel (cached module), the result comes back as "
                         "8 words"},
-        "gpu_launches": 2 * args.steps,
+        # a walk of up to 2,048 32-chunk tasks reduces its own results; beyond, a reduction kernel follows
+        "gpu_launches": args.steps * (1 if GRAY_STEPS >> (first.chunk_log2 + 5) <= 2048 else 2),
         "clocks": {"sm_mhz": clk["sm_mhz"], "sm_max_mhz": clk["sm_max_mhz"], "reasons": clk["reasons"]},
         "plan": {"ms_compile": first.ms_compile, "ms_plan": first.ms_plan, "regs": first.regs_per_thread,
                  "threads": first.threads, "chunk_log2": first.chunk_log2, "reg_rows": first.reg_rows,
