@@ -490,8 +490,9 @@ bool vm_rebuild(perm_plan_s &P) {
 }
 
 static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
+    const bool was = P.use_elim;
     P.vm = P.use_elim = false;
-    adopt_elim(P);
+    if (was) adopt_elim(P);
     const int n = P.m.n;
     if (!elim_allowed(P) || n < min_n || n > 48 || P.opts.engine == PERM_ENGINE_CODEGEN) return false;
     const double range = std::log2((double)(P.g_hi - P.g_lo));

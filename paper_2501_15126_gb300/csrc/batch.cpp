@@ -339,7 +339,7 @@ extern "C" perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, co
         auto work = [&](int t) {
             for (int32_t i = t; i < count; i += nthreads) {
                 plans[i].reset(new perm_plan_s());
-                prep[i] = plan_prepare(&mats[i], &opts, *plans[i], nullptr, 0, true);
+                prep[i] = plan_prepare(&mats[i], &opts, *plans[i], nullptr, 0, mats[i].n >= kVmMinBatch);
                 if (prep[i] == PERM_OK && !plans[i]->zero) vm_prepare(*plans[i], kVmFullBlocksShared, kVmMinBatch);
             }
         };

@@ -47,7 +47,7 @@ struct ElimTable {
     double bound;      // exact: a bound of every entry's magnitude
     int row;           // >= 0: single value x_row (scope empty)
 };
-enum ElimTableKind : uint8_t { kTabRow = 0, kTabMul = 1, kTabSum = 2, kTabSub = 3, kTabProd = 4 };
+enum ElimTableKind : uint8_t { kTabRow = 0, kTabMul = 1, kTabSum = 2, kTabSub = 3 };
 struct ElimTableOp {
     uint8_t kind;
     int dst, a, b;     // row: a = row index

@@ -174,8 +174,11 @@ int range_free_cols(const perm_plan_s &P);
 // again for the plan's current arithmetic (a double-double rerun).
 constexpr double kVmFullBlocks = 8192.0;   // single matrices: outer steps that fill the GPU
 constexpr double kVmFullBlocksShared = 64.0;   // batch and serving: other matrices fill it
-// Below min_n the chained walk takes less time than the planning.
-constexpr int kVmMinBatch = 9, kVmMinServe = 22;   // (a submitter plans alone: 40 us at n = 22)
+// Below min_n the chained walk takes less time than the planning: 200 matrices of
+// n = 10..14 in a batch 2.0 ms chained, 3.6 ms planned; 300 of n = 14..18 3.7 and
+// 3.2 ms, where the chained walk of all of them takes 10.6 ms.  A submitter plans
+// alone, 40 us at n = 22.
+constexpr int kVmMinBatch = 16, kVmMinServe = 22;
 bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n);
 bool vm_rebuild(perm_plan_s &P);
 // Task chunks of a matrix that shares a launch with others: outer steps per lane.

@@ -740,7 +740,7 @@ perm_status_t perm_submit(perm_server_t s, const perm_matrix_t *A, uint64_t *tic
     perm_opts_t po;
     std::memset(&po, 0, sizeof(po));
     po.precision = s->opts.precision;
-    perm_status_t st = plan_prepare(A, &po, *r->P, nullptr, 0, true);
+    perm_status_t st = plan_prepare(A, &po, *r->P, nullptr, 0, A && A->n >= kVmMinServe);
     if (st != PERM_OK) return st;
     perm_plan_s &P = *r->P;
     // a server with a deadline keeps the chained walk, as a call with one does
