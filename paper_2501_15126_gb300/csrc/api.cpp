@@ -1033,8 +1033,15 @@ static perm_status_t compute_one(perm_plan_t plan, void *stream, perm_result_t *
         } else {
             s = plan_launch(*plan, st);
         }
+        // Also after a failure: the upload, or a whole walk, may be queued, and reads
+        // the staging area and the device buffer that the plan gives back when it is
+        // destroyed.  Where the wait fails too, the buffers are not given to another plan.
+        const cudaError_t e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            plan->res.size_class = -1;
+            cudaGetLastError();
+        }
         if (s != PERM_OK) { std::memset(out, 0, sizeof(*out)); out->status = s; return s; }
-        cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { out->status = PERM_ERR_CUDA; return cuda_fail(e, "cudaStreamSynchronize"); }
         plan->computes += 1;
         plan->uploaded = true;

@@ -6,8 +6,9 @@
 // released set goes to a free list of its device and size class and the next
 // plan takes it from there; each list keeps at most kKeep sets (about 10 MB of
 // device memory per device in all), and what does not fit is freed.  A plan holds
-// its set alone from create to destroy, and every compute ends with its stream
-// synchronised, so a released set has no work in flight.
+// its set alone from create to destroy, and every compute, a failed one too, ends
+// with its stream synchronised, so a released set has no work in flight; a set
+// whose stream could not be waited for is freed instead (size_class = -1).
 #pragma once
 
 #include <cstddef>
