@@ -24,6 +24,7 @@
 #include <sstream>
 #include <string>
 #include <unordered_map>
+#include <unordered_set>
 #include <vector>
 
 #include <cuda.h>
@@ -557,7 +558,8 @@ constexpr int kMaxElimFrame = 4096;   // bytes per thread of an eliminated FP64 
 
 std::mutex g_cache_mu;
 std::unordered_map<std::string, CacheEntry> g_cache;
-constexpr size_t kCacheMax = 512;
+std::unordered_set<std::string> g_rejected;   // eliminated steps whose build spills more than it may
+constexpr size_t kCacheMax = 512;             // of each
 
 }  // namespace
 
@@ -700,6 +702,7 @@ perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
     const double t0 = now_ms();
     CacheEntry ce;
     std::string key;
+    bool compiled = false;   // a build of this call's was rejected
     auto cached = [&](const std::string &src) {
         key = "device " + std::to_string(dev) + "\n" + src;
         if (!use_cache) return false;
@@ -712,13 +715,20 @@ perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
         P.cg.blocks_per_sm = it->second.blocks_per_sm;
         P.cg.cached = true;
         P.regs = P.cg.regs;
-        P.ms_compile = 0.0;
+        P.ms_compile = compiled ? now_ms() - t0 : 0.0;
         return true;
+    };
+    auto rejected = [&] {
+        if (!use_cache) return false;
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        return g_rejected.count(key) > 0;
     };
     // The eliminated walk, planned narrower while its kernel spills more than it
     // may (255 registers): FP64 steps have some sixty issue slots per operation
     // of the FP64 pipe, so spills to L1 cost them little; exact ones get none.
-    // Then the chained walk.
+    // Then the chained walk.  A rejected build is remembered: the next plan of the
+    // matrix goes straight on (0/1 n=48 bands: 38 -> 3 ms a plan, and seconds
+    // where the compiler starts cold).
     perm_status_t st = PERM_OK;
     bool built = false;
     for (int width = elim_width(P); width >= 2 && !built; --width) {
@@ -726,6 +736,7 @@ perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
         if (!P.use_elim) break;
         const std::string src = elim_source(P.m, P.elim, P.m.is_int ? P.limbs : 0, P.want_abs);
         if (cached(src)) { adopt_elim(P); return PERM_OK; }
+        if (rejected()) continue;
         st = compile_and_load(src, ce, err, 0);
         if (st != PERM_OK) return st;
         if (ce.local_bytes <= (P.arith == 0 ? kMaxElimFrame : 0)) {
@@ -733,6 +744,9 @@ perm_status_t codegen_build(perm_plan_s &P, std::string &err) {
         } else {
             driver().moduleUnload(ce.module);
             ce = CacheEntry();
+            compiled = true;
+            std::lock_guard<std::mutex> lk(g_cache_mu);
+            if (use_cache && g_rejected.size() < kCacheMax) g_rejected.insert(key);
         }
     }
     P.use_elim = built;
