@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "batch.hpp"
+#include "chunks.hpp"
 #include "plan.hpp"
 
 namespace perm {
@@ -33,7 +34,7 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 int batch_chunk_log2(int n, int B, int K_target) {
     // 32 chunks fill a warp task; keep at least one full task when n allows
-    int K = std::min(K_target, n - 1 - 5);
+    int K = std::min(K_target ? K_target : batch_default_chunk_log2(n), n - 1 - 5);
     K = std::max(K, B);
     return std::min(K, n - 1);
 }
@@ -221,7 +222,8 @@ static perm_status_t run_groups(std::map<std::pair<int, int>, BatchGroup> &group
                 G.img = G.kind == kKindDD ? kImgDD : (G.arith ? kImgInt : kImgF64);
                 autotune_group(G, st);
             }
-            K_target = tuned_chunk_log2(kv.first.first, kv.first.second);
+            if (chunk_log2_is_tuned(kv.first.first, kv.first.second))
+                K_target = tuned_chunk_log2(kv.first.first, kv.first.second);
         }
         perm_status_t s = (perm_status_t)G.setup(kv.first.first, kv.first.second, K_target);
         if (s != PERM_OK) return s;

@@ -13,8 +13,9 @@ struct perm_plan_s;
 
 namespace perm {
 
-// Chunk length (log2) of an n x n matrix in a batch: the group's target,
-// lowered so that the matrix still fills a 32-lane task, never below B.
+// Chunk length (log2) of an n x n matrix in a batch: the group's target (0: the
+// matrix's own, batch_default_chunk_log2), lowered so that the matrix still fills
+// a 32-lane task, never below B.
 int batch_chunk_log2(int n, int B, int K_target);
 
 // The autotuned chunk target of a (NMAX, kernel family) pair (tune.cpp); the

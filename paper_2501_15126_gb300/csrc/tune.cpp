@@ -22,7 +22,7 @@ namespace perm {
 namespace {
 std::mutex g_mu;
 std::map<std::pair<int, int>, int> g_choice;
-constexpr int kDefaultK = 9;   // small groups: a few long chunks would leave most SMs idle
+constexpr int kDefaultK = 12;
 constexpr int kCandidates[] = {8, 10, 12, 14};
 constexpr size_t kSampleMats = 256;
 constexpr size_t kMinMatsToTune = 64;
