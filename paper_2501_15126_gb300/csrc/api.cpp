@@ -14,6 +14,7 @@
 
 #include <cuda_runtime.h>
 
+#include "chunks.hpp"
 #include "codegen.hpp"
 #include "host.hpp"
 #include "kernels.hpp"
@@ -538,12 +539,9 @@ bool vm_prepare(perm_plan_s &P, double full_blocks, int min_n) {
 }
 
 void choose_shared_chunks(perm_plan_s &P, int max_tasks_log2) {
-    const int h = P.elim.h;
-    int K = std::max(0, std::min(3, h - 5));   // 2^3 outer steps a lane, and full warps first
-    K = std::max(K, h - 5 - max_tasks_log2);
-    P.K = K;
+    P.K = shared_chunk_log2(P.elim.h, max_tasks_log2);
     P.chunk_lo = 0;
-    P.chunk_hi = 1ull << (h - K);
+    P.chunk_hi = 1ull << (P.elim.h - P.K);
     P.ntasks = (P.chunk_hi + 31) / 32;
 }
 

@@ -53,7 +53,7 @@ int BatchGroup::setup(int nmax_, int kind_, int K_target) {
     for (size_t i = 0; i < plans.size(); ++i) {
         perm_plan_s &P = *plans[i];
         if (P.vm) {
-            choose_shared_chunks(P, 26);
+            choose_shared_chunks(P, kBatchTasksLog2);
         } else {
             P.K = batch_chunk_log2(P.m.n, gf.block_log2, K_target);
             P.chunk_lo = 0;

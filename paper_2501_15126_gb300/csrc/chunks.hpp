@@ -14,4 +14,13 @@ namespace perm {
 // 27.5 ms at 2^9, 27.1 at 2^10), up to the 2^12 steps of every longer walk.
 inline int batch_default_chunk_log2(int n) { return std::min(12, std::max(9, n - 18)); }
 
+// Eliminated walks that share a launch, h outer columns: 2^3 outer steps a lane, and
+// full warps first; beyond 2^max_tasks_log2 tasks the chunks grow.
+inline int shared_chunk_log2(int h, int max_tasks_log2) {
+    return std::max(std::max(0, std::min(3, h - 5)), h - 5 - max_tasks_log2);
+}
+// A matrix of a batch: up to 1.5 MB of results, dozens of tasks for every warp that
+// the GPU holds (one n=36 p=0.2 FP64: 45.5 ms with 2^20 tasks, 44.2 with 2^16).
+constexpr int kBatchTasksLog2 = 16;
+
 }  // namespace perm
