@@ -3,7 +3,8 @@
 
 #include <map>
 #include <mutex>
-#include <vector>
+
+#include <cuda.h>
 
 namespace perm {
 
@@ -13,11 +14,30 @@ constexpr size_t kClassBytes[] = {64 * 1024, 512 * 1024};   // walks of up to 2^
 constexpr int kClasses = 2;
 constexpr size_t kKeep = 16;
 
+struct FreeList {
+    size_t count = 0;
+    PlanRes set[kKeep];
+};
+
 std::mutex g_mu;
-std::map<std::pair<int, int>, std::vector<PlanRes>> &lists() {
+std::map<std::pair<int, int>, FreeList> &lists() {
     // never destroyed: the CUDA runtime may be gone before static destructors run
-    static auto *l = new std::map<std::pair<int, int>, std::vector<PlanRes>>();
+    static auto *l = new std::map<std::pair<int, int>, FreeList>();
     return *l;
+}
+
+// The id of the allocation at p, 0 if there is none (a context is bound to the thread).
+unsigned long long buffer_id(const void *p) {
+    typedef CUresult (*Fn)(void *, CUpointer_attribute, CUdeviceptr);
+    static const Fn fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q);
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(f) : nullptr;
+    }();
+    unsigned long long id = 0;
+    if (!fn || fn(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return 0;
+    return id;
 }
 
 void release(PlanRes &r) {
@@ -37,11 +57,13 @@ cudaError_t plan_res_take(size_t bytes, PlanRes *out) {
     for (int c = 0; c < kClasses && r.size_class < 0; ++c)
         if (bytes <= kClassBytes[c]) r.size_class = c;
     if (r.size_class >= 0) {
+        if ((e = cudaSetDevice(r.device)) != cudaSuccess) return e;   // binds its context to this thread
         std::lock_guard<std::mutex> lk(g_mu);
-        std::vector<PlanRes> &l = lists()[{r.device, r.size_class}];
-        if (!l.empty()) {
-            *out = l.back();
-            l.pop_back();
+        FreeList &l = lists()[{r.device, r.size_class}];
+        while (l.count) {
+            const PlanRes &s = l.set[--l.count];
+            if (buffer_id(s.dev) != s.buffer_id) continue;   // gone with its context
+            *out = s;
             return cudaSuccess;
         }
     }
@@ -53,6 +75,8 @@ cudaError_t plan_res_take(size_t bytes, PlanRes *out) {
         release(r);
         return e;
     }
+    r.buffer_id = buffer_id(r.dev);
+    if (!r.buffer_id) r.size_class = -1;   // cannot be told from a dead one: not kept
     *out = r;
     return cudaSuccess;
 }
@@ -61,9 +85,9 @@ void plan_res_give(PlanRes &r) {
     if (!r.dev) return;
     if (r.size_class >= 0) {
         std::lock_guard<std::mutex> lk(g_mu);
-        std::vector<PlanRes> &l = lists()[{r.device, r.size_class}];
-        if (l.size() < kKeep) {
-            l.push_back(r);
+        FreeList &l = lists()[{r.device, r.size_class}];
+        if (l.count < kKeep) {
+            l.set[l.count++] = r;
             r = PlanRes();
             return;
         }

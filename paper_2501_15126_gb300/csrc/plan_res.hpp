@@ -8,7 +8,9 @@
 // device memory per device in all), and what does not fit is freed.  A plan holds
 // its set alone from create to destroy, and every compute, a failed one too, ends
 // with its stream synchronised, so a released set has no work in flight; a set
-// whose stream could not be waited for is freed instead (size_class = -1).
+// whose stream could not be waited for is freed instead (size_class = -1).  The
+// sets of a context that cudaDeviceReset ended are gone with it: a listed set is
+// handed out only while the driver still knows its buffer by the id it had.
 #pragma once
 
 #include <cstddef>
@@ -25,6 +27,7 @@ struct PlanRes {
     uint64_t *host = nullptr;        // 8 pinned words, then the staging area
     unsigned char *stage() const { return reinterpret_cast<unsigned char *>(host + 8); }
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    unsigned long long buffer_id = 0;   // the driver's, unique in the process: dev's allocation
 };
 
 constexpr size_t kStageBytes = 32 * 1024;

@@ -1,5 +1,9 @@
 """The device buffer and pinned memory of a plan go on to the next plan when it is
 destroyed: nothing may be in flight on them by then, whatever its calls returned."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 import oracle
@@ -7,6 +11,7 @@ from paper_2501_15126_gb300 import _abi as A
 from paper_2501_15126_gb300 import synth
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("kw", [{"engine": A.PERM_ENGINE_GENERIC}, {"engine": A.PERM_ENGINE_GENERIC, "chunk_log2": 5},
@@ -33,3 +38,27 @@ def test_a_failed_compute_returns_with_its_stream_idle(kw):
         q.close()
     finally:
         A.inject_failures(A.PERM_SITE_LAUNCH, 0)
+
+
+RESET = """
+import ctypes, sys
+from paper_2501_15126_gb300 import _abi as A, synth
+a, b = synth.single_er(14, 0.3, 1, values="01"), synth.single_er(15, 0.3, 2, values="f64")
+def both(**kw):
+    return [A.permanent(m, engine=A.PERM_ENGINE_GENERIC, **kw).value for m in (a, b)]
+want = both() + both(chunk_log2=5)
+kept = [A.Plan(m, engine=A.PERM_ENGINE_GENERIC) for m in (a, b, a, b)]
+for p in kept:
+    p.compute()
+    p.close()
+assert ctypes.CDLL("libcudart.so.13").cudaDeviceReset() == 0
+plans = [A.Plan(m, engine=A.PERM_ENGINE_GENERIC) for m in (a, b, a, b)]
+assert [p.compute().value for p in plans] == want[:2] * 2
+assert both() + both(chunk_log2=5) == want
+"""
+
+
+def test_plans_after_a_device_reset_take_buffers_of_the_new_context():
+    """cudaDeviceReset ends the process's own context and frees what it held; a plan
+    created afterwards gets none of it.  In a process of its own."""
+    subprocess.run([sys.executable, "-c", RESET], cwd=ROOT, check=True, timeout=300)
