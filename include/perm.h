@@ -263,7 +263,8 @@ perm_status_t perm_batch(const perm_matrix_t *mats, int32_t count, const perm_op
    cudaFree).  The paper has no counterpart: it is a packaging of the
    precompiled walk.  Its scratch memory is a file-scope device array of
    1 MiB that every GPU loading the library holds until exit; host
-   temporaries live on the stack.  n <= 48 (PERM_ERR_SIZE beyond), generic
+   temporaries live on the stack (some 60 KB) and, while a call plans, in a
+   file-scope host array that calls take in turn.  n <= 48 (PERM_ERR_SIZE beyond), generic
    kernels only (engine CODEGEN gives PERM_ERR_ARG).  The first call on a
    device looks up the array's device address with that device current, so
    make it before any stream capture.  All calls share the array: two calls

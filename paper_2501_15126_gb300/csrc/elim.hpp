@@ -54,8 +54,8 @@ struct ElimTableOp {
     int col;           // sum, sub: the column's place in the elimination order
 };
 
-// (`mem` is where a plan and its image keep their vectors: the heap, or the stack
-// of the allocation-free call.)
+// (`mem` is where a plan and its image keep their vectors: the heap, or the fixed
+// memory of the allocation-free call.)
 struct ElimPlan {
     explicit ElimPlan(std::pmr::memory_resource *mem = std::pmr::new_delete_resource())
         : ops(mem), bound(mem), tables(mem), tops(mem), factors(mem) {}

@@ -7,8 +7,8 @@
 // precompiled generic walk with its scratch memory (counters, per-task
 // partial sums, the matrix image and the task table) in one file-scope
 // device array instead of device allocations.  It allocates no device or
-// pinned host memory; its host-side temporaries are on the stack or in the
-// plan's host-only bookkeeping.
+// pinned host memory; its host-side temporaries are on the stack (some 60 KB) or,
+// while the walk is planned, in a file-scope host array that calls take in turn.
 //
 // The array is kNoAllocScratchBytes (1 MiB) on every GPU that loads this
 // library and stays allocated until the process exits.  Its device address
@@ -38,7 +38,7 @@ constexpr size_t kOffBatchMat = 192;              // one pk::BatchMat
 constexpr size_t kOffImage = 256;                 // the matrix image (<= 20480 bytes)
 constexpr size_t kImageBytes = 20480;
 constexpr size_t kOffTasks = kOffImage + kImageBytes;   // per-task partial sums
-constexpr size_t kPlannerBytes = 128 * 1024;      // the eliminated walk's plan and program, on the stack
+constexpr size_t kPlannerBytes = 384 * 1024;      // the eliminated walk's plan and program, three widths at the most
 constexpr int kMaxDevices = 64;
 static_assert(sizeof(pk::BatchMat) <= kOffImage - kOffBatchMat, "task table entry");
 // (finish.cuh writes words 1..6 from two words before the result)
@@ -48,6 +48,11 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 
 std::mutex g_mu;
 unsigned char *g_scratch_addr[kMaxDevices] = {};
+
+// Host memory of the planner: one call plans at a time (25-300 us), whatever its
+// device, and is done with it once its image is in the upload.
+std::mutex g_planner_mu;
+alignas(16) unsigned char g_planner[kPlannerBytes];
 
 // The device address of g_noalloc_scratch on the current device.
 perm_status_t scratch_for_current_device(unsigned char **out) {
@@ -85,7 +90,9 @@ int chunk_log2_that_fits(const perm_plan_s &P, uint64_t max_tasks, int K_from) {
 
 // One walk of a prepared plan (FP64, double-double or exact) in the scratch
 // array; fills *out.  Every error return sets out->status too.
-perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream_t st_, perm_result_t *out) {
+// `mem` is the planner's memory, where P keeps its vectors.
+perm_status_t walk_in_scratch(perm_plan_s &P, std::pmr::monotonic_buffer_resource &mem, unsigned char *scratch,
+                              cudaStream_t st_, perm_result_t *out) {
     using namespace perm;
     auto failed = [&](perm_status_t s) { out->status = s; return s; };
     const int n = P.m.n;
@@ -100,9 +107,16 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     size_t img_bytes = 0;
     // the eliminated walk where its image and task results fit the array
     bool vm = false;
-    try {
-        vm = n > 8 && vm_prepare(P, kVmFullBlocks, 9) && P.vm_img.size() <= kImageBytes;
-    } catch (const std::bad_alloc &) {   // the planner's stack is full: the chained walk
+    std::unique_lock<std::mutex> planning(g_planner_mu, std::defer_lock);
+    if (n > 8) {
+        planning.lock();
+        P.elim = ElimPlan(&mem);   // (a first pass's vectors are another call's by now)
+        P.vm_img = std::pmr::vector<unsigned char>(&mem);
+        mem.release();
+        try {
+            vm = vm_prepare(P, kVmFullBlocks, 9) && P.vm_img.size() <= kImageBytes;
+        } catch (const std::bad_alloc &) {   // the planner's memory is full: the chained walk
+        }
     }
     if (vm) {
         P.gf = generic_fns(P.family_nmax(), P.family_kind());
@@ -154,6 +168,7 @@ perm_status_t walk_in_scratch(perm_plan_s &P, unsigned char *scratch, cudaStream
     std::memset(up, 0, kOffImage);
     if (vm) std::memcpy(up + kOffImage, P.vm_img.data(), img_bytes = P.vm_img.size());
     else build_devmat_into(P.m, P.L, P.img_kind(), P.nmax, up + kOffImage);
+    if (planning.owns_lock()) planning.unlock();
     if (!P.direct) {
         pk::BatchMat bm;
         std::memset(&bm, 0, sizeof(bm));
@@ -226,15 +241,13 @@ extern "C" perm_status_t perm_compute_noalloc(const perm_matrix_t *A, const perm
     if (st != PERM_OK) return failed(st);
 
     alignas(16) unsigned char dense[kNoAllocMaxN * kNoAllocMaxN * 8];
-    // the planner's vectors live on the stack too
-    alignas(16) unsigned char planner[kPlannerBytes];
-    std::pmr::monotonic_buffer_resource mem(planner, sizeof(planner), std::pmr::null_memory_resource());
+    std::pmr::monotonic_buffer_resource mem(g_planner, sizeof(g_planner), std::pmr::null_memory_resource());
     perm_plan_s P(&mem);   // host bookkeeping only: nothing on the device is allocated through it
     st = plan_prepare(A, opts, P, dense, sizeof(dense), true);
     if (st != PERM_OK) return failed(st);
     if (P.zero) { describe(P, out); out->status = PERM_OK; return PERM_OK; }
     cudaStream_t st_ = reinterpret_cast<cudaStream_t>(stream);
-    st = walk_in_scratch(P, scratch, st_, out);
+    st = walk_in_scratch(P, mem, scratch, st_, out);
     // precision AUTO: an ill-conditioned whole FP64 walk runs again in
     // double-double, in the same scratch array
     if (st == PERM_OK && !P.m.is_int && !P.dd && !P.subrange && P.opts.precision == PERM_PREC_AUTO &&
@@ -242,7 +255,7 @@ extern "C" perm_status_t perm_compute_noalloc(const perm_matrix_t *A, const perm
         P.dd = true;
         P.direct = false;
         P.opts.chunk_log2 = opts ? opts->chunk_log2 : 0;
-        st = walk_in_scratch(P, scratch, st_, out);
+        st = walk_in_scratch(P, mem, scratch, st_, out);
     }
     return st;
 }

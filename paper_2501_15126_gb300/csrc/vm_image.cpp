@@ -45,23 +45,21 @@ size_t vm_slot_area(int img, int limbs, int nslots, int nextra) {
 }
 
 bool vm_image(const Matrix &m, const ElimPlan &E, int img, int limbs, int max_slots, std::pmr::vector<unsigned char> &out) {
-    // working vectors on the stack, beyond that where the image is
-    alignas(16) unsigned char work[48 * 1024];
-    std::pmr::monotonic_buffer_resource local(work, sizeof(work), out.get_allocator().resource());
+    // working vectors in one block from where the image is (threads of small stacks call this)
+    std::pmr::monotonic_buffer_resource local(48 * 1024, out.get_allocator().resource());
     std::pmr::memory_resource *mem = &local;
     const int n = m.n;
     const bool exact = img == kImgInt;
     const int ntab = (int)E.tables.size();
     const std::pmr::vector<ElimTableOp> &tops = E.tops;
     // literals: the entries that the program and the flips add; literal 0 pads
-    int lit_of[kNMax][kNMax];
-    std::memset(lit_of, -1, sizeof lit_of);
+    std::pmr::vector<short> lit_of((size_t)n * n, -1, mem);
     std::pmr::vector<std::pair<int, int>> lits(1, {-1, -1}, mem);
-    auto lit = [&](int r, int c) {
-        int &l = lit_of[r][c];
+    auto lit = [&](int r, int c) -> int {
+        short &l = lit_of[(size_t)r * n + c];
         if (l >= 0) return l;
         lits.push_back({r, c});
-        return l = (int)lits.size() - 1;
+        return l = (short)(lits.size() - 1);
     };
     // ring tables: 64-bit slots hold what their bound allows (everything, modulo 2^64, in a 64-bit ring)
     auto is_ring = [&](int t) { return exact && limbs > 2 && !(E.tables[t].bound < 9.2e18); };
