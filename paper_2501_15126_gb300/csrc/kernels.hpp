@@ -23,7 +23,7 @@ struct GenericFns {
 // kind = 2 limbs + fold: limbs 0 = FP64 (fold 0) or double-double (fold 1,
 // kKindDD), 2..6 = exact modulo 2^(32 limbs); fold = 1 selects the exact
 // kernels that multiply slot quadruples in 32 bits first (every row's
-// absolute sum <= 127).  nmax in {16, 32, 48}; 1..3 are the eliminated walk's
+// absolute sum <= 127).  nmax in {16, 32, 48}; 1..5 are the eliminated walk's
 // shared-memory classes (vm.hpp), whose exact kinds have fold = 0.
 constexpr int kKindDD = 1;
 GenericFns generic_fns(int nmax, int kind);
