@@ -476,6 +476,7 @@ void codegen_choose_elim(perm_plan_s &P, int max_width) {
     const double range = std::log2((double)(P.g_hi - P.g_lo));
     if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return;
     if (P.elim.ops_per_step > 0.5 * P.ops_per_step) return;
+    if (P.want_abs && !elim_magnitudes_hold(P.m, P.elim, P.L.col_order, range_free_cols(P), P.g_lo, P.g_hi)) return;
     P.use_elim = true;
 }
 
@@ -521,6 +522,7 @@ static bool vm_plan(perm_plan_s &P, double full_blocks, int min_n) {
         if (!elim_plan(P.m, P.L.col_order, range_free_cols(P), range, lim, P.elim)) return false;
         const double steps = std::max(std::exp2(range - P.elim.k), full_blocks);
         if ((P.elim.table_ops + 10.0) * (P.m.is_int ? 10.0 : 1.0) * steps > 0.9 * chain) return false;
+        if (!P.m.is_int && !elim_magnitudes_hold(P.m, P.elim, P.L.col_order, range_free_cols(P), P.g_lo, P.g_hi)) return false;
         P.vm = P.use_elim = true;
         if (vm_rebuild(P)) {
             adopt_elim(P);

@@ -421,7 +421,7 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
         for (int j = 0; j < n; ++j) rs += std::fabs(m.fval(i, j));
         if (!(rs > 0.0) || !std::isfinite(rs)) return false;
         std::frexp(rs / 2.0, &E.exp2[i]);
-        E.exp2[i] -= elim_row_bits(n, k);
+        E.exp2[i] -= elim_row_bits(n, k, i);
         E.scale += E.exp2[i];
     }
     double count;
@@ -436,6 +436,101 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
     for (int p = 0; p < h; ++p) flips += pc(m.colmask[E.outer[p]]) * std::ldexp(1.0, -(p + 1));
     E.ops_per_step = std::ldexp(count + flips + 1.0, -k);
     return true;
+}
+
+bool elim_magnitudes_hold(const Matrix &m, const ElimPlan &E, const int *col_order, int free_cols, uint64_t g_lo,
+                          uint64_t g_hi) {
+    const int n = m.n;
+    free_cols = std::min(free_cols, n - 1);
+    // Scaled rows: |x_i| <= 2^b_i, and a nonzero x_i is at least one unit of the last
+    // place of the row's finest entry, 2^g_i.
+    int g[kNMax], bmin = 1 << 20;
+    double x0[kNMax];
+    for (int i = 0; i < n; ++i) {
+        bmin = std::min(bmin, elim_row_bits(n, E.k, i));
+        g[i] = 1 << 20;
+        double rs = 0.0;
+        for (uint64_t c = m.rowmask[i]; c; c &= c - 1) {
+            const double v = m.fval(i, __builtin_ctzll(c));
+            int e;
+            const int64_t bits = (int64_t)std::ldexp(std::frexp(std::fabs(v), &e), 53);
+            g[i] = std::min(g[i], e - 53 + __builtin_ctzll((uint64_t)bits) - 1 - E.exp2[i]);
+            rs += v;
+        }
+        x0[i] = m.fval(i, E.last) - rs / 2.0;
+    }
+    // the fewest rows whose product may be below FP32's normal numbers
+    insertion_sort(g, g + n, [](int a, int b) { return a < b; });
+    int rows = 0;
+    for (int sum = 0; sum >= -126; sum += g[rows++])
+        if (rows == n) return true;
+    // Each of a step's at most 2^7 tables may lose 2^-150 an entry (a single value
+    // 2^-126: it is cut off there), times the largest magnitudes of the rows that are
+    // still to come and the settings of the low columns: 2^(120 - rows bmin) at most.
+    // The mean step's sum of magnitudes has to be 2^20 times that.
+    const double need = 20.0 + 7.0 + (rows == 1 ? -126.0 : -150.0) + 120.0 - rows * bmin;
+    // It is at least one term of the range over the number of its steps.  The free
+    // columns take every setting: none and all of them (the largest terms of matrices
+    // without negative entries), then each improved column by column.
+    const double floor_log2 = E.k - std::log2((double)(g_hi - g_lo));
+    double x[kNMax];
+    auto fill = [&](uint64_t set) {
+        for (int i = 0; i < n; ++i) {
+            x[i] = x0[i];
+            for (uint64_t c = m.rowmask[i] & set; c; c &= c - 1) x[i] += m.fval(i, __builtin_ctzll(c));
+        }
+    };
+    auto term_log2 = [&] {
+        double mant = 1.0;
+        int exp = 0;
+        for (int i = 0; i < n && mant != 0.0; ++i) {
+            int e;
+            mant = std::frexp(mant * std::fabs(std::ldexp(x[i], -E.exp2[i])), &e);
+            exp += e;
+        }
+        return mant == 0.0 ? -1e300 : exp + std::log2(mant);
+    };
+    auto columns = [&](uint64_t q) {   // the columns set at Gray index q
+        uint64_t set = 0;
+        for (uint64_t u = q ^ (q >> 1); u; u &= u - 1) set |= 1ull << col_order[__builtin_ctzll(u)];
+        return set;
+    };
+    uint64_t free = 0;
+    for (int p = 0; p < free_cols; ++p) free |= 1ull << col_order[p];
+    const uint64_t start[2] = {columns(g_lo) & ~free, columns(g_lo) | free};
+    for (int improve = 0; improve < 2; ++improve)
+        for (uint64_t set : start) {
+            fill(set);
+            for (uint64_t left = improve ? free : 0; left; left &= left - 1) {
+                const int j = __builtin_ctzll(left);
+                const double sign = (set >> j) & 1ull ? -1.0 : 1.0;
+                double now = 1.0, then = 1.0;   // (factors from 2^-20: zeros are left where they can be)
+                for (uint64_t r = m.colmask[j]; r; r &= r - 1) {
+                    const int i = __builtin_ctzll(r);
+                    now *= std::max(std::fabs(std::ldexp(x[i], -E.exp2[i])), 0x1p-20);
+                    then *= std::max(std::fabs(std::ldexp(x[i] + sign * m.fval(i, j), -E.exp2[i])), 0x1p-20);
+                }
+                if (then <= now) continue;
+                set ^= 1ull << j;
+                for (uint64_t r = m.colmask[j]; r; r &= r - 1) x[__builtin_ctzll(r)] += sign * m.fval(__builtin_ctzll(r), j);
+            }
+            if (term_log2() + floor_log2 >= need) return true;
+        }
+    // Last, the mean of sampled |terms|, from below: the largest over the number of samples.
+    uint64_t seed = 0x9e3779b97f4a7c15ull;
+    double top = -1e300;
+    int draws = 0;
+    for (int terms = 0; terms < 8 && draws < 1024; ++draws) {
+        seed += 0x9e3779b97f4a7c15ull;   // splitmix64
+        uint64_t z = seed;
+        z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+        z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+        fill(columns(g_lo + (z ^ (z >> 31)) % (g_hi - g_lo)));
+        const double t = term_log2();
+        if (t > -1e300) ++terms;
+        top = std::max(top, t);
+    }
+    return top - std::log2((double)draws) + E.k >= need;
 }
 
 // ------------------------------------------------------------------ generated kernel

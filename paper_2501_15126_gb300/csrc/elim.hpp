@@ -99,10 +99,23 @@ bool elim_plan(const Matrix &m, const int *col_order, int free_cols, double rang
                ElimPlan &out);
 
 // FP64 rows are scaled by powers of two (exactly) to |x_i| <= 2^bits, so that a
-// product of n of them, summed over 2^(k+3) terms, neither leaves FP32's range
-// (the sum of |terms|) nor drifts into its subnormals, whatever the rows' own
-// magnitudes.
-inline int elim_row_bits(int n, int k) { return std::max(0, std::min(8, (120 - k) / n)); }
+// product of n of them, summed over 2^(k+3) terms, does not leave FP32's range (the
+// sum of |terms|), whatever the rows' own magnitudes; the first rows take what the
+// division leaves over.
+inline int elim_row_bits(int n, int k, int row) {
+    const int b = std::max(0, std::min(8, (120 - k) / n));
+    return b < 8 && row < 120 - k - b * n ? b + 1 : b;
+}
+
+// Whether the magnitudes of FP64 terms, multiplied in FP32 in the program's order,
+// give the sum of |terms| of [g_lo, g_hi).  A product of few rows underflows long
+// before the whole term would (four pairs of rows that cancel to 2^-52 of each other:
+// terms of 2^-208 of the largest possible one, their sum came out as 0 at n = 28),
+// so the sum must stay above what the program's underflows can lose.  It is bounded
+// by terms of the range, or estimated from sampled ones; true where nothing can
+// underflow.
+bool elim_magnitudes_hold(const Matrix &m, const ElimPlan &E, const int *col_order, int free_cols, uint64_t g_lo,
+                          uint64_t g_hi);
 
 // The CUDA C++ of the generated kernel (limbs 0: FP64, else the exact ring).
 std::string elim_source(const Matrix &m, const ElimPlan &E, int limbs, bool want_abs);
