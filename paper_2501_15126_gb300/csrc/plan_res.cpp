@@ -26,18 +26,35 @@ std::map<std::pair<int, int>, FreeList> &lists() {
     return *l;
 }
 
+template <class F>
+F driver_entry(const char *name) {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<F>(f) : nullptr;
+}
+
 // The id of the allocation at p, 0 if there is none (a context is bound to the thread).
 unsigned long long buffer_id(const void *p) {
-    typedef CUresult (*Fn)(void *, CUpointer_attribute, CUdeviceptr);
-    static const Fn fn = [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q);
-        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(f) : nullptr;
-    }();
+    static const auto fn = driver_entry<CUresult (*)(void *, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
     unsigned long long id = 0;
     if (!fn || fn(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return 0;
     return id;
+}
+
+// The thread's context; the device's primary one is bound first where it has none.
+cudaError_t current_context(void **out) {
+    static const auto fn = driver_entry<CUresult (*)(CUcontext *)>("cuCtxGetCurrent");
+    CUcontext c = nullptr;
+    *out = nullptr;
+    if (!fn || fn(&c) != CUDA_SUCCESS) return cudaSuccess;   // unknown: nothing is kept
+    if (!c) {
+        const cudaError_t e = cudaFree(nullptr);
+        if (e != cudaSuccess) return e;
+        fn(&c);
+    }
+    *out = c;
+    return cudaSuccess;
 }
 
 void release(PlanRes &r) {
@@ -57,12 +74,15 @@ cudaError_t plan_res_take(size_t bytes, PlanRes *out) {
     for (int c = 0; c < kClasses && r.size_class < 0; ++c)
         if (bytes <= kClassBytes[c]) r.size_class = c;
     if (r.size_class >= 0) {
-        if ((e = cudaSetDevice(r.device)) != cudaSuccess) return e;   // binds its context to this thread
+        if ((e = current_context(&r.context)) != cudaSuccess) return e;
         std::lock_guard<std::mutex> lk(g_mu);
         FreeList &l = lists()[{r.device, r.size_class}];
-        while (l.count) {
-            const PlanRes &s = l.set[--l.count];
-            if (buffer_id(s.dev) != s.buffer_id) continue;   // gone with its context
+        for (size_t i = l.count; i-- > 0;) {
+            const PlanRes s = l.set[i];
+            const bool alive = buffer_id(s.dev) == s.buffer_id;
+            if (alive && s.context != r.context) continue;   // another context's
+            l.set[i] = l.set[--l.count];                     // taken, or gone with its context
+            if (!alive) continue;
             *out = s;
             return cudaSuccess;
         }
@@ -76,7 +96,7 @@ cudaError_t plan_res_take(size_t bytes, PlanRes *out) {
         return e;
     }
     r.buffer_id = buffer_id(r.dev);
-    if (!r.buffer_id) r.size_class = -1;   // cannot be told from a dead one: not kept
+    if (!r.buffer_id || !r.context) r.size_class = -1;   // cannot be told from a dead one: not kept
     *out = r;
     return cudaSuccess;
 }

@@ -10,7 +10,8 @@
 // with its stream synchronised, so a released set has no work in flight; a set
 // whose stream could not be waited for is freed instead (size_class = -1).  The
 // sets of a context that cudaDeviceReset ended are gone with it: a listed set is
-// handed out only while the driver still knows its buffer by the id it had.
+// handed out only in the context it was made in, while the driver still knows its
+// buffer by the id it had.
 #pragma once
 
 #include <cstddef>
@@ -27,6 +28,7 @@ struct PlanRes {
     uint64_t *host = nullptr;        // 8 pinned words, then the staging area
     unsigned char *stage() const { return reinterpret_cast<unsigned char *>(host + 8); }
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    void *context = nullptr;            // the CUDA context it was made in
     unsigned long long buffer_id = 0;   // the driver's, unique in the process: dev's allocation
 };
 

@@ -62,3 +62,27 @@ def test_plans_after_a_device_reset_take_buffers_of_the_new_context():
     """cudaDeviceReset ends the process's own context and frees what it held; a plan
     created afterwards gets none of it.  In a process of its own."""
     subprocess.run([sys.executable, "-c", RESET], cwd=ROOT, check=True, timeout=300)
+
+
+CONTEXTS = """
+import ctypes
+from paper_2501_15126_gb300 import _abi as A, synth
+cu = ctypes.CDLL("libcuda.so.1")
+a, b = synth.single_er(14, 0.3, 1, values="01"), synth.single_er(15, 0.3, 2, values="f64")
+def both():
+    return [A.permanent(m, engine=A.PERM_ENGINE_GENERIC).value for m in (a, b)]
+want = both()
+ctx, old = ctypes.c_void_p(), ctypes.c_void_p()
+assert cu.cuCtxCreate_v2(ctypes.byref(ctx), 0, 0) == 0       # current from here on
+assert both() == want
+assert cu.cuCtxPopCurrent_v2(ctypes.byref(old)) == 0
+assert both() == want
+assert cu.cuCtxPushCurrent_v2(ctx) == 0
+assert both() == want and both() == want
+assert cu.cuCtxPopCurrent_v2(ctypes.byref(old)) == 0
+"""
+
+
+def test_plans_in_a_context_of_the_callers_own_take_its_buffers():
+    """A driver context beside the device's primary one, by turns."""
+    subprocess.run([sys.executable, "-c", CONTEXTS], cwd=ROOT, check=True, timeout=300)
