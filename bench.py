@@ -38,6 +38,7 @@ sys.path.insert(0, ROOT)
 
 N36 = dict(n=36, p=0.15, seed=2)
 GRAY_STEPS = 1 << 35
+FUSED_TASKS = 2048   # kFusedTasks of csrc/plan.hpp
 NOMINAL_FP64_ISSUE = 2 * 152 * 2.07e9   # 1.25 TFLOP/s nominal = 2 FP64 lane-ops/clk/SM x 152 SMs x 2.07 GHz
 L2_FLUSH_BYTES = 256 << 20              # > 129 MB L2
 METRIC = "Gray-code steps/s (n=36 single sparse matrix permanent)"
@@ -115,12 +116,13 @@ def traffic_record(kernel_hash: str):
 
 def kernel_hash() -> str:
     """Identifies the timed kernel: the CUDA C++ the generator emits for the
-    workload matrix (which fixes its layout and scheme) and the two headers it
-    is compiled with."""
+    workload matrix (the eliminated walk's, the chained walk's where that runs)
+    and the headers it is compiled with."""
     from paper_2501_15126_gb300 import _abi as A
+    a = workload_matrix()
     h = hashlib.sha256()
-    h.update(A.codegen_source(workload_matrix()).encode())
-    for name in ("core.cuh", "devmat.h"):
+    h.update((A.elim_source(a)[0] or A.codegen_source(a)).encode())
+    for name in ("core.cuh", "devmat.h", "finish.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2501_15126_gb300", "csrc", name), "rb").read())
     return h.hexdigest()[:16]
 
@@ -396,8 +398,8 @@ def run_ours(args):
                 "note": "perm_plan_create + perm_compute + perm_plan_destroy from a host CSR matrix; the matrix "
                         "reaches the GPU inside the generated kernel (cached module), the result comes back as "
                         "8 words"},
-        # a walk of up to 2,048 32-chunk tasks reduces its own results; beyond, a reduction kernel follows
-        "gpu_launches": args.steps * (1 if GRAY_STEPS >> (first.chunk_log2 + 5) <= 2048 else 2),
+        # a walk of few 32-chunk tasks reduces its own results; beyond, a reduction kernel follows
+        "gpu_launches": args.steps * (1 if GRAY_STEPS >> (first.chunk_log2 + 5) <= FUSED_TASKS else 2),
         "clocks": {"sm_mhz": clk["sm_mhz"], "sm_max_mhz": clk["sm_max_mhz"], "reasons": clk["reasons"]},
         "plan": {"ms_compile": first.ms_compile, "ms_plan": first.ms_plan, "regs": first.regs_per_thread,
                  "threads": first.threads, "chunk_log2": first.chunk_log2, "reg_rows": first.reg_rows,
