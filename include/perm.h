@@ -190,7 +190,8 @@ typedef struct {
     uint64_t partial[3];
     int32_t exact_words;
     int32_t engine;        /* PERM_ENGINE_GENERIC or PERM_ENGINE_CODEGEN that ran     */
-    int32_t ordering;      /* PERM_ORDER_* that was used                              */
+    int32_t ordering;      /* PERM_ORDER_* that was used (where the chained walk runs: */
+                           /*   the eliminated one orders its own columns)             */
     int32_t reg_rows;      /* k: rows of x in registers                               */
     int32_t reg_cols;      /* c: columns that touch register rows only               */
     int32_t chunk_log2;    /* K                                                       */
@@ -399,16 +400,17 @@ perm_status_t perm_codegen_source(const perm_matrix_t *A, const perm_opts_t *opt
    Writes the source like perm_codegen_source, which gives the chained walk's
    kernel; *len is 0 and *k is 0 where the chained walk runs instead (an explicit
    order, split, chunk length or chain scheme, a deadline, a walk of zero
-   spans, or no column worth summing out).  order (n entries or NULL) gets the
+   spans, magnitudes that would underflow in the program where abs_term_sum is
+   kept, or no column worth summing out).  order (n entries or NULL) gets the
    outer columns by Gray position, then the k low columns, then the last
    column. */
 perm_status_t perm_elim_source(const perm_matrix_t *A, const perm_opts_t *opts, char *buf, int64_t cap,
                                int64_t *len, int32_t *k, int32_t *order);
 
 /* The program image that the precompiled eliminated walk reads for A (for
-   inspection): the same walk as perm_elim_source's, its step written as bundles
-   of four operations on numbered slots (start values, entries, flip lists of
-   the outer columns, program).  shared_launch = 1 plans as perm_batch and the
+   inspection): the same walk as perm_elim_source's, its step written as
+   instructions on whole tables in numbered slots (start values, entries, flip
+   lists of the outer columns, program).  shared_launch = 1 plans as perm_batch and the
    server do, 0 as a plan of its own.  *kind is the arithmetic (0 FP64, 1
    double-double, else 2 limbs), the walk's sum is the true one times 2^-scale
    and its sum of |terms| times 2^-abs_shift; *len is 0 where the chained walk

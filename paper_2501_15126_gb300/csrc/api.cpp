@@ -459,9 +459,10 @@ static void codegen_layout(perm_plan_s &P) {
 }
 
 // Plans the eliminated walk of a generated kernel (tables of at most
-// 2^max_width entries).  Walks whose zero spans skip most of the range keep
-// those: their chained walk drops 87-99.996 % of the steps.  Elsewhere the line is
-// half the chain's counted operations per Gray step: a step's program has no
+// 2^max_width entries).  Walks of zero spans keep the chained walk, which drops
+// 87-99.996 % of their steps; that rule was not drawn from times of both (the
+// counts of the eliminated walk are lower there too).  Elsewhere the line is half
+// the chain's counted operations per Gray step: a step's program has no
 // block start, vote or skip, so equal counts would already be even, and dense
 // patterns (J_30: nothing to share) stay with the chain.  Measured, chained ->
 // eliminated (tables of 2^5 entries): n=36 p=0.15 FP64 368 -> 2.76 ms per

@@ -20,7 +20,7 @@ inline int shared_chunk_log2(int h, int max_tasks_log2) {
     return std::max(std::max(0, std::min(3, h - 5)), h - 5 - max_tasks_log2);
 }
 // A matrix of a batch: up to 1.5 MB of results, dozens of tasks for every warp that
-// the GPU holds (one n=36 p=0.2 FP64: 45.5 ms with 2^20 tasks, 44.2 with 2^16).
+// the GPU holds (one n=36 p=0.2 FP64: 45.5 ms with 2^17 tasks, 44.2 with 2^16).
 constexpr int kBatchTasksLog2 = 16;
 
 }  // namespace perm

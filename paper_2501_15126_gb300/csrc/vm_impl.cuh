@@ -11,7 +11,8 @@
 // hide one another's latency.  The value slots of a warp (10-40 KB) set how many
 // warps an SM holds, so there is one value per lane and slot.
 //
-// Measured (n=28 p=0.3 FP64, 2^27 Gray steps): 1.23 ms, 6 warps per SM; with a
+// Measured (an n=28 p=0.3 FP64 matrix of 3.1 operations per Gray step, 2^27 steps;
+// most of its family count 2.5 and take 0.8-0.9 ms): 1.22 ms, 6 warps per SM; with a
 // range of slots per partial product, 10 % more slots and 5 warps, 1.33 ms at
 // 58 % FP64-pipe activity.  Taken back: scalar instructions in bundles of four, one
 // value per slot, 1.24 ms with 9 % fewer operations (56 % of the pipe); two values
